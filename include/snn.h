@@ -454,6 +454,13 @@ int snn_sim_workspace_bytes(const snn_routing *rt, const snn_sim_params *p, size
  * changes a result, every combination is bit-exact):
  *   SNN_PERSIST=0               CUDA-graph path instead of the persistent kernel
  *   SNN_PERSIST_SMEM=0          persistent kernel on global neuron state only
+ *   SNN_RESIDENT=0              no resident kernel (the whole network on the
+ *                               chip; also off with SNN_PERSIST=0,
+ *                               SNN_PERSIST_SMEM=0, SNN_PERSIST_DEFER=1 and any
+ *                               SNN_PERSIST_BLOCKS_PER_SM or SNN_BAR_GROUPS)
+ *   SNN_RESIDENT_BLOCKS=g       resident kernel on (about) g blocks
+ *   SNN_RESIDENT_THREADS=n      resident kernel with n threads per block
+ *   SNN_RESIDENT_LIST=n         resident kernel with lists of at most n entries
  *   SNN_PERSIST_BLOCKS_PER_SM=b at most b (1..4) resident blocks per SM
  *   SNN_PERSIST_DEFER=1         minimum-delay batching, as defer_delayed = 1
  *   SNN_DELIVERY=0..3           overrides snn_sim_params.delivery
@@ -518,7 +525,14 @@ int snn_batch_create(const snn_network *net, const snn_routing *rt, int32_t n, c
  * grid barrier after each half, each barrier wait bounded by one second);
  * otherwise, or with the environment variable SNN_PERSIST=0 at
  * snn_sim_create, as replays of captured CUDA graphs of two kernels per
- * step.  Both give the same results bit for bit.
+ * step.  Both give the same results bit for bit.  With SNN_DELIVER_RING or
+ * _AUTO, a network whose pending input (4 bytes per neuron and step of the
+ * largest delay) fits in the SMs' shared memory runs in the resident kernel
+ * instead, also one launch for T steps: neuron state, delay ring and exchange
+ * fill counters stay on the chip, a block has one bounded wait per step (for
+ * the spikes of the others).  Its tables, a copy of the synapses ordered by
+ * target block, are part of the workspace; with a workspace that has no room
+ * for them the network runs as above.
  * Errors raised on the device are reported by snn_sync_status.
  * Errors: SNN_E_ARG, SNN_E_CUDA.
  */
@@ -583,8 +597,8 @@ int snn_sim_reset(snn_sim *sim, int32_t reupload);
  * persistent kernel with 4, 3, 2 or 1 blocks per SM and the neuron state in
  * shared memory, in global memory with 16-byte accesses or one neuron per
  * thread, the CUDA-graph path, each with delivery into the delay ring and
- * (workspace of SNN_DELIVER_AUTO) by arrival step, and the partition-owned
- * kernel -- each from the sim's current state, and keep the fastest (shapes
+ * (workspace of SNN_DELIVER_AUTO) by arrival step, the partition-owned
+ * kernel and the resident kernel -- each from the sim's current state, and keep the fastest (shapes
  * excluded by SNN_PERSIST=0 / SNN_PERSIST_SMEM=0 at creation are not
  * tried).  Every shape gives the same results bit for bit.  The exchange
  * capacities need no tuning: they are the exact worst case of the routing
@@ -593,7 +607,7 @@ int snn_sim_reset(snn_sim *sim, int32_t reupload);
  * choice (may be NULL): 0 = graph path, else 100 * mode + blocks per SM
  * (mode 2 shared-memory state, 1 global 16-byte, 0 global one neuron per
  * thread), + 1000 with delivery by arrival step; 2000 + blocks per SM for
- * the partition-owned kernel; best_ms (may be NULL): the chosen shape's time
+ * the partition-owned kernel; 3001 for the resident kernel; best_ms (may be NULL): the chosen shape's time
  * per step.  Synchronises the stream.  Host memory: a copy of the neuron
  * state and the delay ring.
  * Errors: SNN_E_ARG, SNN_E_CUDA.
@@ -675,6 +689,9 @@ int64_t snn_launches(const snn_sim *sim, int32_t T);
  * arrival step), [3] the rest of the wait at the first grid barrier, [4] the
  * routing walk (a4-a5), [5] the routing rounds' deliveries and copies (a6),
  * [6] the next step's input-free update and the wait at the second barrier.
+ * Resident kernel (block 0's step warps): [0] update, [1] publication of the
+ * spikes, [2] the next step's drive, [3] gather, [4] and [5] delivery, [6] the
+ * step's end (routing and raster run beside them).
  * Graph path: [0] the k_update kernel and [4] the k_route kernel of every
  * step (CUDA events between them, which add a little time), the rest 0.
  * Synchronises the stream.  Errors: SNN_E_ARG, SNN_E_CUDA.

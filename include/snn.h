@@ -631,12 +631,14 @@ int snn_autotune(snn_sim *sim, int32_t steps, int32_t *choice, double *best_ms);
  * Rates r_a = (spikes of population a) / (T N_a).  Backward: surrogate
  * dS/dV_pre = 1 / (1 + beta |V_pre - V_th|)^2, reset detached; each neuron
  * gathers its targets' adjoints along its own level-2 entries (the
- * transpose of the routed delivery).  Backward step t gathers the newest
- * adjoint plane only, h(t + 1) = G[pop k][b] * dL/dV_pre of k at t + 1, and
- * adds each synapse's term to a per-step partial sum by its delay; the
- * float32 terms are summed in a fixed order per neuron, so the gradients do
- * not depend on the checkpoint interval.  Gradients are accumulated in
- * float64 (per-warp float pairs first).
+ * transpose of the routed delivery).  Networks of 25,000 neurons or more gather
+ * the adjoints of up to three steps at once (a synapse of delay d contributes d
+ * steps earlier, so those of delay >= 3 are read every third step), smaller
+ * ones step by step; the float32 terms are summed in a fixed order per neuron,
+ * so the gradients do not depend on the checkpoint interval.  Gradients are
+ * accumulated as float pairs and added in float64.  The environment variable
+ * SNN_ADJ_BATCHED=0|1, read by snn_adjoint_workspace_bytes and
+ * snn_adjoint_create, selects one of the two (tests).
  */
 typedef struct {
     int32_t T;            /* forward steps per run (>= 1) */

@@ -21,17 +21,21 @@
 // level-2 entries and synapse segments (the transpose of the routed
 // delivery), and the parameter gradients accumulate in float64.
 //
-// Backward step t gathers only the newest adjoint plane, that of step t + 1,
-// and spreads each synapse's term over the step it belongs to, t + 1 - d, in
-// per-delay partial sums (a neuron's sum for step t is complete once step
-// t + 1 has been gathered).  So the gather reads one plane of n_pop x M
-// floats, and the slice of the source's own partition (most targets) is
-// staged in shared memory.  Every segment's steps run as one CUDA graph
-// whose kernels read the segment's first step from device memory.
+// The term of a synapse (j -> k, delay d) of step t is w G[pop k][pop j] g_k(t +
+// d), g the adjoint of V_pre.  The synapses of delay d >= 3 are read every
+// third step only, when the planes of three steps are complete, and gather the
+// three at once (for the steps d earlier); delay 2 every second step two,
+// delay 1 every step one: 0.44 of the synapses per step for delays uniform in
+// 1..8, and one index per three gathered planes.  The planes are
+// kept interleaved (three or two steps of a neuron in one 16- or 8-byte word),
+// the slice of a source's own partition (most targets) staged in shared
+// memory.  Every segment's steps run as one CUDA graph whose kernels read the
+// segment's first step from device memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <new>
@@ -46,17 +50,24 @@ namespace {
 constexpr int kAThreads = 256;
 constexpr int kBThreads = 1024;  // backward: one block per SM, up to 64 registers (32 warps hide latency)
 constexpr int kBWarps = kBThreads / 32;
-constexpr int kBGroups = 2;      // groups of 4 synapses per lane per batch (a run of 256 in one batch)
+constexpr int kBGroups = 2;      // k_adj_backward_runs: groups of 4 synapses per lane per batch
+constexpr int kBUnroll = 8;      // synapses of a source in flight
+constexpr int64_t kBatchedNeurons = 25000;  // see adj_batched
+constexpr int kParts = 2;        // parts of a partition staged one after the other; other targets are part kParts
+constexpr int kKinds = kParts + 1;
+constexpr int kBatch = 3;        // steps gathered at once by a synapse of delay >= kBatch
+constexpr int kItemSources = 1024;  // sources per work unit, at most (their sums are in shared memory)
 constexpr int kDWarps = 4;       // forward delivery: warps per spike
 constexpr int kDUnroll = 4;
 constexpr int kMaxPop = 8;
 constexpr uint32_t kNoiseTag = 0xAD;
 
 // A backward block's unit of work: sources j0..j1-1 of one partition, whose
-// first n_stage neurons (from base) are staged for planes plane0, plane0+1.
+// first n_stage neurons (from base) are staged, cap of them at a time; slices
+// of 32 sources from sl0.
 struct BItem {
     uint32_t j0, j1, base, n_stage;
-    uint32_t plane0, pad0, pad1, pad2;
+    uint32_t sl0, n_sl, plane0, pad;  // (plane0: first plane of the partition's VN, k_adj_backward_runs)
 };
 
 struct AdjDev {
@@ -90,12 +101,25 @@ struct AdjDev {
     uint8_t *seg_flag;      // [K][M] bit 0 spike, bit 1 refractory
     int32_t *seg_A;         // [K][M][n_pop]
     // backward
-    float *hbuf;            // [2][n_pop][M] by step parity: G[pop k][b] * (adjoint of V_pre of k);
-                            // a source of population b gathers plane b
-    float *part;            // [S][M] partial sums of the gathered terms, by step slot (step mod S)
-    int S;                  // step slots = largest delay
+    // The backward's synapses, by item, kind (part of the source's partition
+    // that holds the target, or none), delay, slice of 32 sources; inside a slice column k holds the k-th synapse of every source that
+    // has one, so a lane per source reads whole columns.
+    uint2 *rec;             // [E] target | pop << 28, float bits of w G[pop of target][pop of source]
+    const int16_t *rec_w;   // [E] the weights in that order
+    const uint32_t *cnt;    // [kKinds S M] synapses by (item, kind, delay, source)
+    const unsigned long long *col;  // [kKinds S slices] first record of each (item, kind, delay, slice)
+    // k_adj_backward_runs: planes [2][n_pop][M] by step parity, G[pop k][b] * (adjoint of V_pre of k); partial sums
+    // [S][M] by step slot
+    float *hbuf, *rpart;
+    float *g1;              // [2][M] adjoint of V_pre by step parity
+    float2 *g2;             // [2][M] the same of steps 2 m, 2 m + 1 (m mod 2)
+    float4 *g3;             // [2][M] the same of steps 3 m .. 3 m + 2 (m mod 2)
+    float *part;            // [R][M] gathered terms of steps to come (step mod R)
+    float2 *gacc;           // [n_pop + 1][M] float pairs: a neuron's sums of g c A_b and of g c w_ext
+    int S, R;               // largest delay; steps a step's gathers reach (at least 2)
     const BItem *items;     // [n_items] backward work units
-    int n_items, cap;       // staged neurons per plane (shared memory)
+    int n_items, cap, src_cap;  // neurons staged at a time, sources per item (shared memory)
+    int ways;               // warps that share a slice's delays
     const int *tb;          // first step of the running segment
     float *gV;              // [M]
     const float *direct;    // [n_pop] dL/dr_a / (T N_a)
@@ -122,6 +146,14 @@ __device__ __forceinline__ uint4 philox_ctr(uint32_t k0, uint32_t k1, uint32_t c
     return make_uint4(x0, x1, x2, x3);
 }
 
+// Programmatic dependent launch (the kernels of a segment's graph): wait for
+// the kernel before this one, let the next one be scheduled early.
+__device__ __forceinline__ void pdl_enter()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ int byte_sum(uint32_t w)
 {
     return (int)(w & 0xFFu) + (int)((w >> 8) & 0xFFu) + (int)((w >> 16) & 0xFFu) + (int)(w >> 24);
@@ -142,6 +174,7 @@ __device__ __forceinline__ float noise_of(const AdjDev &a, uint32_t g, uint32_t 
 template <int NP>
 __global__ void __launch_bounds__(kAThreads) k_adj_update(const AdjDev a, int toff, int rec, int count)
 {
+    pdl_enter();
     const int t = *a.tb + toff;
     __shared__ unsigned long long s_cnt[kMaxPop];
     if (threadIdx.x < kMaxPop) s_cnt[threadIdx.x] = 0;
@@ -211,6 +244,7 @@ __global__ void __launch_bounds__(kAThreads) k_adj_update(const AdjDev a, int to
 // to the ring slot of its delay, column = the source population.
 __global__ void __launch_bounds__(kAThreads) k_adj_deliver(const AdjDev a, int toff)
 {
+    pdl_enter();
     const int t = *a.tb + toff;
     const int par = t & 1;
     const unsigned int n = *(volatile unsigned int *)&a.spk_n[par];
@@ -243,6 +277,348 @@ __global__ void __launch_bounds__(kAThreads) k_adj_deliver(const AdjDev a, int t
 }
 
 // A float sum kept as an unevaluated pair hi + lo (Dekker / Knuth two-sum):
+// adds the exact product gd * x (two-product with one fused multiply-add) and
+// keeps the rounding errors in lo, so hi + lo carries about 48 significant
+// bits.  The float64 pipe of this GPU is slow, so the per-neuron terms stay in
+// the float pipe; k_adj_reduce adds the pairs in float64.
+__device__ __forceinline__ float2 pair_add(float2 a, float gd, float x)
+{
+    const float p = __fmul_rn(gd, x);
+    const float q = __fmaf_rn(gd, x, -p);  // p + q == gd * x exactly
+    const float s = __fadd_rn(a.x, p);
+    const float bp = __fsub_rn(s, a.x);
+    const float err = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bp)), __fsub_rn(p, bp));
+    return make_float2(s, __fadd_rn(a.y, __fadd_rn(err, q)));
+}
+
+// Places of an item's entries in cnt and col.
+__device__ __forceinline__ size_t cnt_at(const AdjDev &a, const BItem &it, int kind, int d)
+{
+    return (size_t)kKinds * a.S * it.j0 + ((size_t)kind * a.S + (d - 1)) * (it.j1 - it.j0);
+}
+
+__device__ __forceinline__ size_t col_at(const AdjDev &a, const BItem &it, int kind, int d, uint32_t sl)
+{
+    return (size_t)kKinds * a.S * it.sl0 + ((size_t)kind * a.S + (d - 1)) * it.n_sl + sl;
+}
+
+// Build the backward's synapse order (targets and weights).  A block per
+// item.  The k-th synapse of a source is the k-th of its kind in the table's
+// order, so the sums' rounding does not change from run to run.
+__global__ void __launch_bounds__(kAThreads) k_adj_sort(const AdjDev a, uint2 *rec, int16_t *rec_w, uint32_t *cnt,
+                                                        unsigned long long *col)
+{
+    constexpr int kW = kAThreads / 32;
+    __shared__ uint32_t s_n[kW][kKinds * kMaxDelay];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nk = kKinds * a.S;
+    uint32_t *n = s_n[wid];
+    for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+        const BItem it = a.items[item];
+        const uint32_t ns = it.j1 - it.j0;
+        auto key = [&](uint32_t td) {
+            const uint32_t rel = (td & kTgtMask) - it.base;
+            return (rel < it.n_stage ? (int)(rel / (uint32_t)a.cap) : kParts) * a.S + (int)(td >> kTgtBits);
+        };
+        for (uint32_t si = wid; si < ns; si += kW) {
+            const unsigned long long r0 = a.run[it.j0 + si], r1 = a.run[it.j0 + si + 1];
+            for (int k = lane; k < nk; k += 32) n[k] = 0u;
+            __syncwarp();
+            for (unsigned long long x = r0 + lane; x < r1; x += 32) atomicAdd(&n[key(a.syn_td[x])], 1u);
+            __syncwarp();
+            for (int k = lane; k < nk; k += 32) cnt[cnt_at(a, it, 0, 1 + k) + si] = n[k];
+            __syncwarp();
+        }
+        __syncthreads();
+        const uint32_t ne = (uint32_t)nk * it.n_sl;  // entries of col, (kind, delay, slice) in order
+        unsigned long long *co = col + col_at(a, it, 0, 1, 0);
+        for (uint32_t e = wid; e < ne; e += kW) {
+            const uint32_t sl = e % it.n_sl, si = sl * 32 + lane;
+            const uint32_t c = si < ns ? cnt[cnt_at(a, it, 0, 1 + (int)(e / it.n_sl)) + si] : 0u;
+            unsigned long long v = c;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+            if (lane == 0) co[e] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned long long at = a.run[it.j0];
+            for (uint32_t e = 0; e < ne; ++e) {
+                const unsigned long long c = co[e];
+                co[e] = at;
+                at += c;
+            }
+        }
+        __syncthreads();
+        for (uint32_t si = wid; si < ns; si += kW) {
+            const unsigned long long r0 = a.run[it.j0 + si], r1 = a.run[it.j0 + si + 1];
+            const uint32_t sl = si >> 5, in = si & 31u, left = min(32u, ns - sl * 32);
+            for (int k = lane; k < nk; k += 32) n[k] = 0u;
+            __syncwarp();
+            for (unsigned long long x0 = r0; x0 < r1; x0 += 32) {
+                const unsigned long long x = x0 + lane;
+                const uint32_t td = x < r1 ? a.syn_td[x] : 0u;
+                const int k = x < r1 ? key(td) : -1;
+                const uint32_t same = __match_any_sync(0xFFFFFFFFu, k);
+                const uint32_t rank = __popc(same & ((1u << lane) - 1u));
+                uint32_t c = 0;
+                if (k >= 0) c = n[k] + rank;
+                __syncwarp();
+                if (k >= 0) {
+                    if (rank == 0) n[k] += __popc(same);
+                    // column c of the slice: the columns before it, the sources before this one in it
+                    const uint32_t *len = cnt + cnt_at(a, it, 0, 1 + k) + sl * 32;
+                    unsigned long long pos = co[(size_t)k * it.n_sl + sl];
+                    for (uint32_t u = 0; u < left; ++u) {
+                        const uint32_t m = len[u];
+                        pos += min(m, c) + (u < in && m > c ? 1u : 0u);
+                    }
+                    const uint32_t t = td & kTgtMask;
+                    rec[pos].x = t | (uint32_t)a.pop[t] << kTgtBits;
+                    rec_w[pos] = a.syn_w[x];
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// The records' factors w G[pop of target][pop of source] for the gains of the
+// forward: a warp per (kind, delay, slice) of an item, column by column.
+__global__ void __launch_bounds__(kAThreads) k_adj_factors(const AdjDev a)
+{
+    __shared__ float s_G[kMaxPop * kMaxPop];
+    const int np = a.n_pop, lane = threadIdx.x & 31;
+    if (threadIdx.x < np * np) s_G[threadIdx.x] = a.G[threadIdx.x];
+    __syncthreads();
+    for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+        const BItem it = a.items[item];
+        for (uint32_t e = threadIdx.x >> 5; e < (uint32_t)(kKinds * a.S) * it.n_sl; e += kAThreads / 32) {
+            const uint32_t sl = e % it.n_sl, si = sl * 32 + lane;
+            const uint32_t len = si < it.j1 - it.j0 ? a.cnt[cnt_at(a, it, 0, 1 + (int)(e / it.n_sl)) + si] : 0u;
+            const int pj = si < it.j1 - it.j0 ? a.pop[it.j0 + si] : 0;
+            unsigned long long at = a.col[col_at(a, it, 0, 1, 0) + e];
+#pragma unroll 4
+            for (uint32_t k = 0, m; (m = __ballot_sync(0xFFFFFFFFu, len > k)) != 0u; ++k) {
+                if (len > k) {
+                    const unsigned long long x = at + __popc(m & ((1u << lane) - 1u));
+                    a.rec[x].y = __float_as_uint(__fmul_rn((float)a.rec_w[x], s_G[(a.rec[x].x >> kTgtBits) * np + pj]));
+                }
+                at += __popc(m);
+            }
+        }
+    }
+}
+
+// One backward step t = (segment start) + toff, segment slot rec.  A block
+// takes the sources of an item.  For the planes that are complete at step t
+// (the last one always: delay 1; two at odd t: delay 2; three when t + 1 is a
+// multiple of 3: delays from 3) a warp takes a slice of 32 sources, a lane per
+// source, and walks the columns of those delays: first the targets in the
+// parts of its own partition, each part's slice of the planes staged in shared
+// memory for the block, then the other targets from global memory.  The sums
+// go to the steps t, t - 1, .. of the source (acc, carried in part).  Step t's
+// sum is then complete and a thread per source runs the adjoint recursion,
+// writes the plane entries of step t and adds the parameter-gradient terms to
+// the neuron's own pairs.
+//
+// The gathers from global memory are bound by the lines that L1 can hold in
+// flight: staging half a partition at a time (98 KB) instead of all of it (196
+// KB) leaves four times as many.  Measured at the adjoint workload (131,072
+// neurons, 500 synapses, delays 1-8): 99 us per step against 191 for
+// k_adj_backward_runs; 132 with the whole partition staged.
+template <int B>
+__device__ __forceinline__ void adj_gather(const AdjDev &a, const BItem &it, int d0, int d1, const float *h1,
+                                           const float2 *h2, const float4 *h3, float *hs, float *acc)
+{
+    const uint32_t ns = it.j1 - it.j0;
+    const int lane = threadIdx.x & 31;
+    const uint32_t cap = (uint32_t)a.cap, stride = cap + 1u, ways = (uint32_t)a.ways;
+#pragma unroll 1
+    for (int kind = 0; kind < kKinds; ++kind) {
+        const uint32_t from = (uint32_t)kind * cap;  // first staged neuron of the part
+        if (kind < kParts && from >= it.n_stage) continue;
+        if (kind < kParts) {
+            const uint32_t n = min(cap, it.n_stage - from);
+            __syncthreads();
+#pragma unroll 4
+            for (uint32_t x = threadIdx.x; x < n; x += kBThreads) {
+                const uint32_t j = it.base + from + x;
+                if constexpr (B == 1) {
+                    hs[x] = h1[j];
+                } else if constexpr (B == 2) {
+                    const float2 v = h2[j];
+                    hs[x] = v.x;
+                    hs[stride + x] = v.y;
+                } else {
+                    const float4 v = h3[j];
+                    hs[x] = v.x;
+                    hs[stride + x] = v.y;
+                    hs[2 * stride + x] = v.z;
+                }
+            }
+            // (a plane's last entry stays 0: what a lane without a synapse multiplies)
+            if (threadIdx.x < B) hs[threadIdx.x * stride + cap] = 0.0f;
+            __syncthreads();
+        }
+        // a warp per slice; with few slices several, which share the delays (each with sums of its own)
+        for (uint32_t wu = threadIdx.x >> 5; wu < it.n_sl * ways; wu += kBThreads / 32) {
+            const uint32_t sl = wu / ways, way = wu - sl * ways;
+            const uint32_t si = sl * 32 + lane;
+            if (d0 + (int)way > d1) continue;
+            // synapses of a delay and their first records, those of the next delay in flight
+            uint32_t n0 = 0;
+            unsigned long long c0;
+            auto bounds = [&](int d) {
+                if (si < ns) n0 = a.cnt[cnt_at(a, it, kind, d) + si];
+                c0 = a.col[col_at(a, it, kind, d, sl)];
+            };
+            bounds(d0 + (int)way);
+#pragma unroll 1
+            for (int d = d0 + (int)way; d <= d1; d += (int)ways) {
+                const uint32_t n = n0;
+                const uint2 *r = a.rec + c0;
+                if (d + (int)ways <= d1) {
+                    bounds(d + (int)ways);
+                    // the slice's records of the next delay into L2
+                    const uint32_t tot = __reduce_add_sync(0xFFFFFFFFu, n0);
+                    for (uint32_t x = 16u * lane; x < tot; x += 512u)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.rec + c0 + x));
+                }
+                float sum[B];
+#pragma unroll
+                for (int b = 0; b < B; ++b) sum[b] = 0.0f;
+                const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n);
+#pragma unroll 1
+                for (uint32_t k = 0; k < most; k += kBUnroll) {
+                    // records of columns [k, k + kBUnroll) (none past a source's last)
+                    uint2 q[kBUnroll];
+#pragma unroll
+                    for (int u = 0; u < kBUnroll; ++u) {
+                        const bool in = n > k + u;
+                        const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+                        q[u] = in ? __ldcs(r + __popc(m & ((1u << lane) - 1u)))
+                                  : make_uint2(it.base + from + cap, 0u);
+                        r += __popc(m);
+                    }
+                    if (kind < kParts) {
+#pragma unroll
+                        for (int u = 0; u < kBUnroll; ++u) {
+                            const float *h = hs + ((q[u].x & kTgtMask) - it.base - from);
+#pragma unroll
+                            for (int b = 0; b < B; ++b)
+                                sum[b] = __fmaf_rn(__uint_as_float(q[u].y), h[b * stride], sum[b]);
+                        }
+                    } else {
+                        float v[kBUnroll][B];
+#pragma unroll
+                        for (int u = 0; u < kBUnroll; ++u) {
+                            const uint32_t x = q[u].x & kTgtMask;
+#pragma unroll
+                            for (int b = 0; b < B; ++b) v[u][b] = 0.0f;
+                            if (n <= k + u) continue;
+                            if constexpr (B == 1) {
+                                v[u][0] = __ldg(h1 + x);
+                            } else if constexpr (B == 2) {
+                                const float2 w = __ldg(h2 + x);
+                                v[u][0] = w.x;
+                                v[u][1] = w.y;
+                            } else {
+                                const float4 w = __ldg(h3 + x);
+                                v[u][0] = w.x;
+                                v[u][1] = w.y;
+                                v[u][2] = w.z;
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < kBUnroll; ++u)
+#pragma unroll
+                            for (int b = 0; b < B; ++b)
+                                sum[b] = __fmaf_rn(__uint_as_float(q[u].y), v[u][b], sum[b]);
+                    }
+                }
+                // the last of the planes is gathered by step t - (d - d0), the one before it by the step before
+                if (si < ns)
+#pragma unroll
+                    for (int b = 0; b < B; ++b)
+                        acc[((int)way * a.R + d - d0 + B - 1 - b) * a.src_cap + si] += sum[b];
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, int toff, int rec)
+{
+    extern __shared__ __align__(16) float bsm[];
+    pdl_enter();
+    const int t = *a.tb + toff;
+    const long long M = a.M;
+    const int np = a.n_pop, R = a.R;
+    float *hs = bsm;                       // [kBatch][cap + 1] staged planes
+    float *acc = bsm + kBatch * (a.cap + 1);    // [ways][R][src_cap] sums of steps t, t - 1, ..
+    const float c = 0.0009765625f;
+    const bool triple = a.S >= kBatch && (t + 1) % kBatch == 0;  // planes t + 1 .. t + 3 are complete
+    const int nacc = triple ? R : 2;       // steps that get terms
+    for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
+        const BItem it = a.items[item];
+        const uint32_t ns = it.j1 - it.j0;
+        __syncthreads();
+        for (int i = 0; i < nacc; ++i)
+            for (uint32_t x = threadIdx.x; x < ns; x += kBThreads)
+                acc[i * a.src_cap + x] = t >= i ? a.part[(size_t)((t - i) % R) * M + it.j0 + x] : 0.0f;
+        for (int x = R * a.src_cap + threadIdx.x; x < a.ways * R * a.src_cap; x += kBThreads) acc[x] = 0.0f;
+        adj_gather<1>(a, it, 1, 1, a.g1 + (size_t)((t + 1) & 1) * M, nullptr, nullptr, hs, acc);
+        if (a.S >= 2 && (t & 1))
+            adj_gather<2>(a, it, 2, 2, nullptr, a.g2 + (size_t)(((t + 1) / 2) & 1) * M, nullptr, hs, acc);
+        if (triple)
+            adj_gather<3>(a, it, 3, a.S, nullptr, nullptr, a.g3 + (size_t)(((t + 1) / kBatch) & 1) * M, hs, acc);
+        __syncthreads();
+        if (a.ways > 1) {
+            for (int x = threadIdx.x; x < nacc * a.src_cap; x += kBThreads)
+                for (int w = 1; w < a.ways; ++w) acc[x] += acc[w * R * a.src_cap + x];
+            __syncthreads();
+        }
+        for (int i = 1; i < nacc; ++i)
+            for (uint32_t x = threadIdx.x; x < ns; x += kBThreads)
+                if (t >= i) a.part[(size_t)((t - i) % R) * M + it.j0 + x] = acc[i * a.src_cap + x];
+        for (uint32_t x = threadIdx.x; x < ns; x += kBThreads) {
+            const uint32_t j = it.j0 + x;
+            const int pj = a.pop[j];
+            const uint8_t fl = a.seg_flag[(long long)rec * M + j];
+            const float vpre = a.seg_vpre[(long long)rec * M + j];
+            float g = 0.0f;
+            if (!(fl & 2)) {
+                const float gS = __fadd_rn(a.direct[pj], __fmul_rn(c, acc[x]));
+                const float dv = __fsub_rn(vpre, a.v_th);
+                const float den = __fadd_rn(1.0f, __fmul_rn(a.beta, fabsf(dv)));
+                const float sg = __frcp_rn(__fmul_rn(den, den));
+                const float keep = (fl & 1) ? 0.0f : a.gV[j];
+                g = __fadd_rn(keep, __fmul_rn(gS, sg));
+            }
+            a.gV[j] = __fmul_rn(a.alpha, g);
+            a.g1[(size_t)(t & 1) * M + j] = g;
+            reinterpret_cast<float *>(a.g2 + (size_t)((t / 2) & 1) * M + j)[t & 1] = g;
+            reinterpret_cast<float *>(a.g3 + (size_t)((t / kBatch) & 1) * M + j)[t % kBatch] = g;
+            // step t's slot is step t - R's from now on
+            a.part[(size_t)(t % R) * M + j] = 0.0f;
+            // parameter-gradient terms g c A_b and g c w_ext: exact products on the neuron's float pairs
+            if (g != 0.0f) {
+                const float gd = __fmul_rn(g, c);
+                const int32_t *A = a.seg_A + ((long long)rec * M + j) * np;
+                for (int b = 0; b < np; ++b) {
+                    const int32_t xi = A[b];
+                    if (xi < (1 << 24) && xi > -(1 << 24))
+                        a.gacc[(size_t)b * M + j] = pair_add(a.gacc[(size_t)b * M + j], gd, (float)xi);
+                    else
+                        atomicAdd(&a.dG[pj * np + b], (double)g * (double)c * (double)xi);
+                }
+                a.gacc[(size_t)np * M + j] = pair_add(a.gacc[(size_t)np * M + j], gd, a.w_ext);
+            }
+        }
+    }
+}
+
+// A float sum kept as an unevaluated pair hi + lo (Dekker / Knuth two-sum):
 // add() takes the exact product gd * x (two-product with one fused
 // multiply-add) and keeps the rounding errors in lo, so hi + lo carries about
 // 48 significant bits; flush() adds hi + lo in float64 and clears the pair.
@@ -269,7 +645,7 @@ struct FloatPairSum {
 };
 
 // One backward step t = (segment start) + toff, segment slot rec, for every
-// neuron, a warp each.  The warp of source j walks j's synapse run (the
+// neuron, a warp each (networks too small for k_adj_backward, see adj_batched).  The warp of source j walks j's synapse run (the
 // transpose of the routed delivery) and takes, for every synapse (k, d),
 // w * h_k(t + 1) from plane pop(j) of step t + 1: a term of j's input adjoint
 // at step t + 1 - d.  The terms collect per lane and delay in shared memory,
@@ -281,9 +657,10 @@ struct FloatPairSum {
 // shared memory; a warp's next source has its run bounds and first batch of
 // synapses in flight while the current source finishes.
 template <int NDL>
-__global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, int toff, int rec)
+__global__ void __launch_bounds__(kBThreads, 1) k_adj_backward_runs(const AdjDev a, int toff, int rec)
 {
     extern __shared__ __align__(16) float bsm[];
+    pdl_enter();
     __shared__ double s_dG[kMaxPop * kMaxPop];
     __shared__ double s_dl[kMaxPop];
     const int t = *a.tb + toff;
@@ -364,7 +741,7 @@ __global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, i
                 n1 = a.run[jn + 1];
                 pn = a.pop[jn];
             }
-            const float pin = holder ? a.part[(size_t)slot * M + j] : 0.0f;
+            const float pin = holder ? a.rpart[(size_t)slot * M + j] : 0.0f;
             const int32_t Ab = lane < np ? a.seg_A[((long long)rec * M + j) * np + lane] : 0;
             const float Gb = lane < np ? a.G[pj * np + lane] : 0.0f;
             uint8_t fl = 0;
@@ -424,7 +801,7 @@ __global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, i
             const float sum = __fadd_rn(pin, r[0]);
             // step t's slot is consumed (and cleared for step t - S); the
             // earlier steps' slots take their terms
-            if (holder) a.part[(size_t)slot * M + j] = dd == 0 ? 0.0f : sum;
+            if (holder) a.rpart[(size_t)slot * M + j] = dd == 0 ? 0.0f : sum;
             float gvp = 0.0f;
             if (lane == 0 && !(fl & 2)) {
                 const float gS = __fadd_rn(dir, __fmul_rn(c, sum));
@@ -470,6 +847,31 @@ __global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, i
     if (threadIdx.x < np && s_dl[threadIdx.x] != 0.0) atomicAdd(&a.dlam[threadIdx.x], s_dl[threadIdx.x]);
 }
 
+// The parameter gradients: every neuron's pairs in float64 by population
+// (blockIdx.y: the column, n_pop for the drive rates).
+__global__ void __launch_bounds__(kAThreads) k_adj_reduce(const AdjDev a)
+{
+    __shared__ double s[kMaxPop];
+    if (threadIdx.x < kMaxPop) s[threadIdx.x] = 0.0;
+    __syncthreads();
+    const int col = blockIdx.y, np = a.n_pop;
+    const float2 *g = a.gacc + (size_t)col * a.M;
+    double v = 0.0;
+    int p = -1;
+    for (long long j = (long long)blockIdx.x * kAThreads + threadIdx.x; j < a.M; j += (long long)gridDim.x * kAThreads) {
+        const int pj = a.pop[j];
+        if (pj != p) {
+            if (p >= 0) atomicAdd(&s[p], v);
+            p = pj;
+            v = 0.0;
+        }
+        v += (double)g[j].x + (double)g[j].y;
+    }
+    if (p >= 0) atomicAdd(&s[p], v);
+    __syncthreads();
+    if (threadIdx.x < np) atomicAdd(col < np ? &a.dG[threadIdx.x * np + col] : &a.dlam[threadIdx.x], s[threadIdx.x]);
+}
+
 __global__ void k_adj_set_step(int *tb, int t)
 {
     *tb = t;
@@ -481,10 +883,12 @@ struct Region {
 
 struct ALayout {
     Region V, ref, ring, pop, gid, run, syn_td, syn_w, spk, spk_n, pop_cnt, raster, raster_n;
-    Region G, lam, seg_vpre, seg_flag, seg_A, hbuf, part, items, tb, gV, direct, dG, dlam;
+    Region G, lam, seg_vpre, seg_flag, seg_A, rec, rec_w, cnt, col, hbuf, rpart, g1, g2, g3, part, gacc, items, tb, gV, direct, dG, dlam;
     Region ck_V, ck_ref, ck_ring;  // [n_ckpt] checkpoints
     size_t total = 0;
-    int D = 2, n_pop = 2, n_ckpt = 1, S = 1, n_items = 1;
+    int D = 2, n_pop = 2, n_ckpt = 1, S = 1, R = 2, n_items = 1;
+    int64_t n_slices = 0;
+    bool batched = false;  // k_adj_backward, else k_adj_backward_runs
 };
 
 void aplace(ALayout &L, Region &r, size_t bytes)
@@ -510,34 +914,50 @@ int sm_count()
     return std::max(1, sms);
 }
 
-// The backward's work units: every partition cut into chunks of sources,
-// about one chunk per SM in all (at least one per partition).  Returns the
-// count; fills `out` when given (n_stage is capped at create).
-int backward_items(const snn_routing *rt, std::vector<BItem> *out)
+// The backward's work units: every partition cut into chunks of at most
+// kItemSources sources, about one chunk per SM in all (at least one per
+// partition).  Returns the count and the slices of 32 sources; fills `out` when given (n_stage is capped at create).
+int backward_items(const snn_routing *rt, std::vector<BItem> *out, int64_t *slices)
 {
     const int sms = sm_count();
     const int64_t M = rt->M;
-    const int32_t s = rt->P / rt->n_vn;
     int n = 0;
+    *slices = 0;
     for (int32_t ip = 0; ip < rt->P; ++ip) {
         const int64_t a = rt->pbase[ip], b = rt->pbase[ip + 1];
         if (b <= a) continue;
-        const int64_t c = std::max<int64_t>(1, (int64_t)sms * (b - a) / std::max<int64_t>(1, M));
+        const int64_t c = std::max<int64_t>((b - a + kItemSources - 1) / kItemSources,
+                                            (int64_t)sms * (b - a) / std::max<int64_t>(1, M));
         for (int64_t x = 0; x < c; ++x) {
-            if (out) {
-                BItem it;
-                std::memset(&it, 0, sizeof(it));
-                it.j0 = (uint32_t)(a + (b - a) * x / c);
-                it.j1 = (uint32_t)(a + (b - a) * (x + 1) / c);
-                it.base = (uint32_t)a;
-                it.n_stage = (uint32_t)(b - a);
-                it.plane0 = (uint32_t)(2 * (ip / s));
-                out->push_back(it);
-            }
+            BItem it;
+            std::memset(&it, 0, sizeof(it));
+            it.j0 = (uint32_t)(a + (b - a) * x / c);
+            it.j1 = (uint32_t)(a + (b - a) * (x + 1) / c);
+            it.base = (uint32_t)a;
+            it.n_stage = (uint32_t)(b - a);
+            it.plane0 = (uint32_t)(2 * (ip / (rt->P / rt->n_vn)));
+            it.sl0 = (uint32_t)*slices;
+            it.n_sl = (it.j1 - it.j0 + 31) / 32;
+            *slices += it.n_sl;
+            if (out) out->push_back(it);
             ++n;
         }
     }
     return std::max(1, n);
+}
+
+// Whether the backward batches steps (k_adj_backward) or walks every run each
+// step (k_adj_backward_runs).  A batched step has several phases in a row, each
+// some loads deep; they pay from about 25,000 neurons.  Measured, forward and
+// backward of 100 steps in ms, runs / batched: 4,096 neurons x 64 synapses
+// 3.1 / 3.4; 20,000 x 300 5.2 / 5.6; 30,000 x 100 4.9 / 4.6; 60,000 x 80 6.9 /
+// 5.3; 100,000 x 60 10.8 / 6.0; 131,072 x 500 22.3 / 14.2.  SNN_ADJ_BATCHED=0|1
+// overrides (tests).
+bool adj_batched(const snn_routing *rt)
+{
+    const char *e = std::getenv("SNN_ADJ_BATCHED");
+    if (e && (e[0] == '0' || e[0] == '1')) return e[0] == '1';
+    return rt->M >= kBatchedNeurons;
 }
 
 int adj_layout(const snn_routing *rt, const snn_sim_params *p, const snn_adjoint_params *ap, ALayout &L)
@@ -546,7 +966,8 @@ int adj_layout(const snn_routing *rt, const snn_sim_params *p, const snn_adjoint
     L = ALayout();
     L.D = rt->max_delay + 1;
     L.S = std::max(1, (int)rt->max_delay);
-    L.n_items = backward_items(rt, nullptr);
+    L.R = std::max(2, L.S);
+    L.n_items = backward_items(rt, nullptr, &L.n_slices);
     L.n_pop = 2 * rt->n_vn;
     if (L.n_pop > kMaxPop) return SNN_E_RANGE;
     L.n_ckpt = (ap->T + ap->ckpt_every - 1) / ap->ckpt_every;
@@ -558,8 +979,7 @@ int adj_layout(const snn_routing *rt, const snn_sim_params *p, const snn_adjoint
     aplace(L, L.pop, M);
     aplace(L, L.gid, rt->identity ? 0 : sizeof(uint32_t) * M);
     aplace(L, L.run, sizeof(unsigned long long) * (M + 1));
-    // the backward reads synapses in aligned groups of 4: up to 3 past the
-    // end, zero-filled (target 0, delay 1, weight 0)
+    // (k_adj_backward_runs reads synapses in aligned groups of 4: up to 3 past the end, zero-filled)
     aplace(L, L.syn_td, sizeof(uint32_t) * (E + 4));
     aplace(L, L.syn_w, sizeof(int16_t) * (E + 4));
     aplace(L, L.spk, sizeof(uint32_t) * 2 * M);
@@ -572,8 +992,21 @@ int adj_layout(const snn_routing *rt, const snn_sim_params *p, const snn_adjoint
     aplace(L, L.seg_vpre, sizeof(float) * (size_t)K * M);
     aplace(L, L.seg_flag, (size_t)K * M);
     aplace(L, L.seg_A, sizeof(int32_t) * (size_t)K * M * L.n_pop);
-    aplace(L, L.hbuf, sizeof(float) * 2 * (size_t)L.n_pop * M);
-    aplace(L, L.part, sizeof(float) * (size_t)L.S * M);
+    L.batched = adj_batched(rt);
+    if (L.batched) {
+        aplace(L, L.rec, sizeof(uint2) * (size_t)E);
+        aplace(L, L.rec_w, sizeof(int16_t) * (size_t)E);
+        aplace(L, L.cnt, sizeof(uint32_t) * (size_t)M * kKinds * L.S);
+        aplace(L, L.col, sizeof(unsigned long long) * kKinds * L.S * (size_t)L.n_slices);
+        aplace(L, L.g1, sizeof(float) * 2 * M);
+        aplace(L, L.g2, sizeof(float2) * 2 * M);
+        aplace(L, L.g3, sizeof(float4) * 2 * M);
+        aplace(L, L.part, sizeof(float) * (size_t)L.R * M);
+        aplace(L, L.gacc, sizeof(float2) * (size_t)(L.n_pop + 1) * M);
+    } else {
+        aplace(L, L.hbuf, sizeof(float) * 2 * (size_t)L.n_pop * M);
+        aplace(L, L.rpart, sizeof(float) * (size_t)L.S * M);
+    }
     aplace(L, L.items, sizeof(BItem) * (size_t)L.n_items);
     aplace(L, L.tb, sizeof(int));
     aplace(L, L.gV, sizeof(float) * M);
@@ -598,8 +1031,8 @@ struct snn_adjoint {
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;  // graph capture
     unsigned grid_n = 1, grid_w = 1, grid_b = 1;
-    int ndl = 8;                        // delay columns of the backward (8 or 16)
-    size_t bsmem = 0;                   // its dynamic shared memory
+    size_t bsmem = 0;                   // dynamic shared memory of the backward
+    int ndl = 8;                        // delay columns of k_adj_backward_runs (8 or 16)
     std::vector<double> pop_size;
     bool have_forward = false;
     // one graph per (kind, segment length): 0 forward counted, 1 forward
@@ -704,9 +1137,19 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
     d.seg_vpre = (float *)(w + L.seg_vpre.off);
     d.seg_flag = (uint8_t *)(w + L.seg_flag.off);
     d.seg_A = (int32_t *)(w + L.seg_A.off);
+    d.rec = (uint2 *)(w + L.rec.off);
+    d.rec_w = (const int16_t *)(w + L.rec_w.off);
+    d.cnt = (const uint32_t *)(w + L.cnt.off);
+    d.col = (const unsigned long long *)(w + L.col.off);
+    d.g1 = (float *)(w + L.g1.off);
+    d.g2 = (float2 *)(w + L.g2.off);
+    d.g3 = (float4 *)(w + L.g3.off);
+    d.gacc = (float2 *)(w + L.gacc.off);
     d.hbuf = (float *)(w + L.hbuf.off);
+    d.rpart = (float *)(w + L.rpart.off);
     d.part = (float *)(w + L.part.off);
     d.S = L.S;
+    d.R = L.R;
     d.items = (const BItem *)(w + L.items.off);
     d.tb = (const int *)(w + L.tb.off);
     d.gV = (float *)(w + L.gV.off);
@@ -753,39 +1196,63 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
     const int sms = sm_count();
     a->grid_n = (unsigned)std::max<int64_t>(1, std::min<int64_t>((M + kAThreads - 1) / kAThreads, 65535));
     a->grid_w = (unsigned)std::max(1, sms * 8);
-    // backward: the delay columns, then as much of each partition's two
-    // planes as shared memory holds
+    // backward: the sums of an item's sources, then as much of a partition's
+    // slice of three planes as shared memory holds
     {
         std::vector<BItem> items;
-        backward_items(rt, &items);
-        a->ndl = rt->max_delay <= 8 ? 8 : 16;
+        int64_t slices = 0;
+        backward_items(rt, &items, &slices);
         int dev = 0, optin = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
             delete a;
             return SNN_E_CUDA;
         }
-        // shared memory: the delay columns, then as much of a partition's two
-        // planes as fits
-        const size_t cols = sizeof(float) * (size_t)kBWarps * a->ndl * 32;
-        const size_t fixed = sizeof(double) * (kMaxPop * kMaxPop + kMaxPop) + 1024;
-        int64_t cap = 0;
-        if ((size_t)optin > cols + fixed) cap = (int64_t)(((size_t)optin - cols - fixed) / (2 * sizeof(float))) & ~3ll;
-        int64_t widest = 0;
-        for (const BItem &it : items) widest = std::max<int64_t>(widest, it.n_stage);
-        cap = std::min<int64_t>(cap, (widest + 3) & ~3ll);
-        for (BItem &it : items) it.n_stage = (uint32_t)std::min<int64_t>(it.n_stage, cap);
-        d.cap = (int)cap;
+        int64_t widest = 0, most = 0;
+        for (const BItem &it : items) {
+            widest = std::max<int64_t>(widest, it.n_stage);
+            most = std::max<int64_t>(most, it.j1 - it.j0);
+        }
         d.n_items = (int)items.size();
-        a->bsmem = cols + 2 * sizeof(float) * (size_t)cap;
-        cudaError_t e = a->ndl == 8 ? cudaFuncSetAttribute(k_adj_backward<8>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a->bsmem)
-                                    : cudaFuncSetAttribute(k_adj_backward<16>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a->bsmem);
-        if (e != cudaSuccess || (int)items.size() != L.n_items ||
+        const void *fn;
+        if (L.batched) {
+            d.ways = (int)std::max<int64_t>(1, std::min<int64_t>(8, kBThreads / std::max<int64_t>(32, (most + 31) / 32 * 32)));
+            const size_t sums = sizeof(float) * (size_t)d.ways * L.R * (size_t)most, fixed = 1024;
+            // (parts of at most 8192 neurons, 96 KB of staged planes: the rest of the SM's memory is L1's, for the
+            // gathers from global memory)
+            int64_t cap = std::min<int64_t>(8192, (int64_t)(((size_t)optin - sums - fixed) / (kBatch * sizeof(float))) - 1);
+            cap = std::min<int64_t>(cap, widest);
+            for (BItem &it : items) it.n_stage = (uint32_t)std::min<int64_t>(it.n_stage, kParts * cap);
+            d.cap = (int)cap;
+            d.src_cap = (int)most;
+            a->bsmem = sums + sizeof(float) * kBatch * (size_t)(cap + 1);
+            fn = (const void *)k_adj_backward;
+        } else {
+            // the delay columns, then as much of a partition's two planes as fits
+            a->ndl = rt->max_delay <= 8 ? 8 : 16;
+            const size_t cols = sizeof(float) * (size_t)kBWarps * a->ndl * 32;
+            const size_t fixed = sizeof(double) * (kMaxPop * kMaxPop + kMaxPop) + 1024;
+            int64_t cap = 0;
+            if ((size_t)optin > cols + fixed) cap = (int64_t)(((size_t)optin - cols - fixed) / (2 * sizeof(float))) & ~3ll;
+            cap = std::min<int64_t>(cap, (widest + 3) & ~3ll);
+            for (BItem &it : items) it.n_stage = (uint32_t)std::min<int64_t>(it.n_stage, cap);
+            d.cap = (int)cap;
+            a->bsmem = cols + 2 * sizeof(float) * (size_t)cap;
+            fn = a->ndl == 8 ? (const void *)k_adj_backward_runs<8> : (const void *)k_adj_backward_runs<16>;
+        }
+        if ((int)items.size() != L.n_items ||
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a->bsmem) != cudaSuccess ||
             cudaMemcpy(w + L.items.off, items.data(), sizeof(BItem) * items.size(), cudaMemcpyHostToDevice) !=
                 cudaSuccess ||
             cudaStreamCreateWithFlags(&a->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+            delete a;
+            return SNN_E_CUDA;
+        }
+        if (L.batched)
+            k_adj_sort<<<(unsigned)std::max(1, d.n_items), kAThreads, 0, a->stream>>>(
+                d, d.rec, (int16_t *)(w + L.rec_w.off), (uint32_t *)(w + L.cnt.off),
+                (unsigned long long *)(w + L.col.off));
+        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(a->stream) != cudaSuccess) {
             delete a;
             return SNN_E_CUDA;
         }
@@ -819,27 +1286,42 @@ static int adj_segment(snn_adjoint *a, int kind, int len)
     if (!ex) {
         cudaStream_t cs = a->cap_stream;
         ACK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        for (int i = 0; i < len; ++i) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.stream = cs;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaError_t le = cudaSuccess;
+        for (int i = 0; i < len && le == cudaSuccess; ++i) {
+            cfg.dynamicSmemBytes = 0;
+            cfg.blockDim = dim3(kAThreads);
             if (kind == 2) {
                 const int toff = len - 1 - i;
-                if (a->ndl == 8)
-                    k_adj_backward<8><<<a->grid_b, kBThreads, a->bsmem, cs>>>(a->dev, toff, toff);
-                else
-                    k_adj_backward<16><<<a->grid_b, kBThreads, a->bsmem, cs>>>(a->dev, toff, toff);
+                cfg.gridDim = dim3(a->grid_b);
+                cfg.blockDim = dim3(kBThreads);
+                cfg.dynamicSmemBytes = a->bsmem;
+                if (a->L.batched) le = cudaLaunchKernelEx(&cfg, k_adj_backward, a->dev, toff, toff);
+                else if (a->ndl == 8) le = cudaLaunchKernelEx(&cfg, k_adj_backward_runs<8>, a->dev, toff, toff);
+                else le = cudaLaunchKernelEx(&cfg, k_adj_backward_runs<16>, a->dev, toff, toff);
             } else {
                 const int rec = kind == 1 ? i : -1, cnt = kind == 0 ? 1 : 0;
+                cfg.gridDim = dim3(a->grid_n);
                 switch (a->dev.n_pop) {
-                case 2: k_adj_update<2><<<a->grid_n, kAThreads, 0, cs>>>(a->dev, i, rec, cnt); break;
-                case 4: k_adj_update<4><<<a->grid_n, kAThreads, 0, cs>>>(a->dev, i, rec, cnt); break;
-                case 6: k_adj_update<6><<<a->grid_n, kAThreads, 0, cs>>>(a->dev, i, rec, cnt); break;
-                default: k_adj_update<8><<<a->grid_n, kAThreads, 0, cs>>>(a->dev, i, rec, cnt); break;
+                case 2: le = cudaLaunchKernelEx(&cfg, k_adj_update<2>, a->dev, i, rec, cnt); break;
+                case 4: le = cudaLaunchKernelEx(&cfg, k_adj_update<4>, a->dev, i, rec, cnt); break;
+                case 6: le = cudaLaunchKernelEx(&cfg, k_adj_update<6>, a->dev, i, rec, cnt); break;
+                default: le = cudaLaunchKernelEx(&cfg, k_adj_update<8>, a->dev, i, rec, cnt); break;
                 }
-                k_adj_deliver<<<a->grid_w, kAThreads, 0, cs>>>(a->dev, i);
+                cfg.gridDim = dim3(a->grid_w);
+                if (le == cudaSuccess) le = cudaLaunchKernelEx(&cfg, k_adj_deliver, a->dev, i);
             }
         }
         cudaGraph_t g = nullptr;
         const cudaError_t e = cudaStreamEndCapture(cs, &g);
-        if (e != cudaSuccess || !g) {
+        if (le != cudaSuccess || e != cudaSuccess || !g) {
+            if (g) cudaGraphDestroy(g);
             a->graphs.erase(std::make_pair(kind, len));
             return SNN_E_CUDA;
         }
@@ -912,8 +1394,15 @@ extern "C" int snn_adjoint_backward(snn_adjoint *a, const double *grates, double
     float direct[kMaxPop] = {0};
     for (int b = 0; b < np; ++b) direct[b] = (float)(grates[b] / ((double)T * a->pop_size[b]));
     ACK(cudaMemcpyAsync(w + L.direct.off, direct, sizeof(direct), cudaMemcpyHostToDevice, st));
-    ACK(cudaMemsetAsync(w + L.hbuf.off, 0, L.hbuf.bytes, st));
-    ACK(cudaMemsetAsync(w + L.part.off, 0, L.part.bytes, st));
+    if (L.batched) {
+        // (g1 .. gacc are one range: planes from step T on and all sums are 0)
+        ACK(cudaMemsetAsync(w + L.g1.off, 0, L.gacc.off + L.gacc.bytes - L.g1.off, st));
+        k_adj_factors<<<(unsigned)a->dev.n_items, kAThreads, 0, st>>>(a->dev);
+        ACK(cudaGetLastError());
+    } else {
+        ACK(cudaMemsetAsync(w + L.hbuf.off, 0, L.hbuf.bytes, st));
+        ACK(cudaMemsetAsync(w + L.rpart.off, 0, L.rpart.bytes, st));
+    }
     ACK(cudaMemsetAsync(w + L.gV.off, 0, L.gV.bytes, st));
     ACK(cudaMemsetAsync(w + L.dG.off, 0, L.dG.bytes, st));
     ACK(cudaMemsetAsync(w + L.dlam.off, 0, L.dlam.bytes, st));
@@ -933,6 +1422,10 @@ extern "C" int snn_adjoint_backward(snn_adjoint *a, const double *grates, double
         if (rc == SNN_OK) rc = adj_segment(a, 2, t1 - t0);
         if (rc != SNN_OK) return rc;
     }
+    if (L.batched)
+        k_adj_reduce<<<dim3((unsigned)std::max(1, std::min(64, (int)((M + kAThreads - 1) / kAThreads))), np + 1), kAThreads, 0,
+                   st>>>(a->dev);
+    ACK(cudaGetLastError());
     ACK(cudaMemcpyAsync(dG, w + L.dG.off, sizeof(double) * np * np, cudaMemcpyDeviceToHost, st));
     ACK(cudaMemcpyAsync(dlam, w + L.dlam.off, sizeof(double) * np, cudaMemcpyDeviceToHost, st));
     ACK(cudaStreamSynchronize(st));

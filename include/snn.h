@@ -712,8 +712,8 @@ int snn_profile_phases(snn_sim *sim, int32_t T, double *phase_ms);
  *   neuron order, accumulated into (the call does not clear it); both
  *   caller-owned.  counts (host uint64 [3], may be NULL) receives the
  *   level-1 entries, level-2 entries and synaptic events of this call.
- * Scratch: the level-1 bucket and level-2 inbox regions of the sim's
- * workspace, so the call must not overlap snn_step on the same sim.
+ * A spike's level-2 entries tile its synapse run, which is delivered as one;
+ * its entries are counted.  The call must not overlap snn_step on the same sim.
  * Runs on the sim's stream, with the sim's device current (the caller's
  * current device is restored), and synchronises the stream before returning.
  * Errors: SNN_E_ARG (n < 0, NULL pointers with n > 0, an id >= M),

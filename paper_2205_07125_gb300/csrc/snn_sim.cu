@@ -244,6 +244,9 @@ static int64_t step_grid(int64_t M)
     return std::max<int64_t>(1, (items + kThreads - 1) / kThreads);
 }
 
+// Largest control word + counters + state read back through page-locked memory.
+constexpr size_t kBackState = (size_t)4 << 20;
+
 // Tally rows: one per block of either launch shape (a persistent grid is
 // capped to the rows there are).
 constexpr int64_t kMinTallyRows = 2048;
@@ -668,6 +671,10 @@ struct snn_sim {
     int test_skip_arrival = 0;  // tests of the bounded wait (SNN_TEST_SKIP_BARRIER)
     std::vector<uint2> row_h;   // the uploaded per-neuron rows (host copy, kept for re-uploads)
     std::vector<void *> pinned;
+    // page-locked host memory of the small read-backs (control word, counters, state): a copy into it is one
+    // transfer without staging by the driver
+    char *back = nullptr;
+    size_t back_bytes = 0;
     // batches: the network of each quad and each network's drive (host copies)
     std::vector<uint16_t> net_of_h;
     std::vector<NetDrive> net_drive_h;
@@ -877,6 +884,7 @@ extern "C" void snn_sim_destroy(snn_sim *s)
     for (cudaEvent_t e : s->pev) cudaEventDestroy(e);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     for (void *p : s->pinned) cudaHostUnregister(p);
+    if (s->back) cudaFreeHost(s->back);
     delete s;
 }
 
@@ -1359,6 +1367,16 @@ static int sim_create(const snn_network *net, const snn_routing *rt, const snn_s
         s->static_row_l1 = m1;
         s->static_row_l2 = m2;
     }
+    {
+        // room for the tally rows, and for control word, counters and state of networks of up to 4 MB of it
+        const size_t state = L.ref.off + L.ref.bytes - L.ctrl.off;
+        s->back_bytes = std::max<size_t>(L.tally.bytes + L.counters.bytes, state <= kBackState ? state : 0);
+        if (cudaHostAlloc((void **)&s->back, s->back_bytes, cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();
+            s->back = nullptr;  // (pageable copies then)
+            s->back_bytes = 0;
+        }
+    }
     rc = upload_tables(s);
     if (!rc) rc = reset_state(s);
     if (rc) {
@@ -1720,8 +1738,9 @@ static int run_fanout(snn_sim *s, FoArgs a, uint64_t *counts)
         k_fanout<<<(unsigned)std::min<long long>(s->grid_fanout, blocks), kThreads, 0, st>>>(a);
         CK(cudaGetLastError());
     }
-    unsigned long long c[4];
-    CK(cudaMemcpyAsync(c, a.cnt, sizeof(c), cudaMemcpyDeviceToHost, st));
+    unsigned long long pageable[4];
+    unsigned long long *c = s->back_bytes >= sizeof(pageable) ? (unsigned long long *)s->back : pageable;
+    CK(cudaMemcpyAsync(c, a.cnt, sizeof(pageable), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (counts)
         for (int k = 0; k < 3; ++k) counts[k] = c[k];
@@ -1829,8 +1848,10 @@ extern "C" int64_t snn_launches_per_step(const snn_sim *s)
 
 static int read_ctrl(snn_sim *s, Ctrl *c)
 {
-    CK(cudaMemcpyAsync(c, s->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s->stream));
+    void *to = s->back_bytes >= sizeof(Ctrl) ? (void *)s->back : (void *)c;
+    CK(cudaMemcpyAsync(to, s->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
+    if (to != c) std::memcpy((void *)c, to, sizeof(Ctrl));
     return SNN_OK;
 }
 
@@ -1900,8 +1921,14 @@ extern "C" int snn_read_raster(snn_sim *s, int64_t t0, int64_t t1, uint32_t *ids
     if (t1 > c.rec_steps) return SNN_E_CAPACITY;
     const int64_t nst = t1 - t0;
     std::vector<long long> off((size_t)nst + 1);
-    CK(cudaMemcpy(off.data(), s->dev.raster_off + t0, sizeof(long long) * (size_t)(nst + 1),
-                  cudaMemcpyDeviceToHost));
+    const size_t off_bytes = sizeof(long long) * (size_t)(nst + 1);
+    if (s->back_bytes >= off_bytes) {
+        CK(cudaMemcpyAsync(s->back, s->dev.raster_off + t0, off_bytes, cudaMemcpyDeviceToHost, s->stream));
+        CK(cudaStreamSynchronize(s->stream));
+        std::memcpy(off.data(), s->back, off_bytes);
+    } else {
+        CK(cudaMemcpy(off.data(), s->dev.raster_off + t0, off_bytes, cudaMemcpyDeviceToHost));
+    }
     const int64_t tot = off[nst] - off[0];
     *n = tot;
     for (int64_t k = 0; k <= nst; ++k) step_off[k] = off[k] - off[0];
@@ -1979,13 +2006,20 @@ extern "C" int snn_read_hashes(snn_sim *s, int64_t t0, int64_t t1, uint64_t *cur
 static int read_counters(snn_sim *s, unsigned long long *c)
 {
     const Layout &L = s->L;
-    std::vector<unsigned long long> rows((size_t)L.tally_rows * C_N);
-    CK(cudaMemcpyAsync(c, s->dev.counters, sizeof(unsigned long long) * C_N, cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(rows.data(), s->dev.tally, sizeof(unsigned long long) * rows.size(), cudaMemcpyDeviceToHost,
-                       s->stream));
+    const size_t nr = (size_t)L.tally_rows * C_N, rb = sizeof(unsigned long long) * nr,
+                 cb = sizeof(unsigned long long) * C_N;
+    std::vector<unsigned long long> pageable;
+    unsigned long long *rows = (unsigned long long *)s->back;
+    if (s->back_bytes < rb + cb) {
+        pageable.resize(nr + C_N);
+        rows = pageable.data();
+    }
+    CK(cudaMemcpyAsync(rows, s->dev.tally, rb, cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(rows + nr, s->dev.counters, cb, cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
-    for (int64_t r = 0; r < L.tally_rows; ++r)
-        for (int k = 0; k < C_N; ++k) c[k] += rows[(size_t)r * C_N + k];
+    for (int k = 0; k < C_N; ++k) c[k] = rows[nr + k];
+    for (size_t r = 0; r < nr; r += C_N)
+        for (int k = 0; k < C_N; ++k) c[k] += rows[r + k];
     return SNN_OK;
 }
 
@@ -2012,15 +2046,37 @@ extern "C" int snn_read_counts(snn_sim *s, snn_counts *o)
 extern "C" int snn_read_state(snn_sim *s, float *V, uint8_t *ref, int64_t *t)
 {
     if (!s) return SNN_E_ARG;
+    const Layout &L = s->L;
     const int64_t M = s->rt->M;
     const uint32_t *inv = s->rt->perm_inv.data();
+    const bool same = s->rt->identity;
+    const size_t span = L.ref.off + L.ref.bytes - L.ctrl.off;
+    if (s->back_bytes >= span) {
+        // control word, counters, potentials and refractory counters lie together: one copy
+        CK(cudaMemcpyAsync(s->back, s->ws + L.ctrl.off, span, cudaMemcpyDeviceToHost, s->stream));
+        CK(cudaStreamSynchronize(s->stream));
+        const float *v = (const float *)(s->back + (L.V.off - L.ctrl.off));
+        const uint8_t *r = (const uint8_t *)(s->back + (L.ref.off - L.ctrl.off));
+        if (V && same) std::memcpy(V, v, sizeof(float) * (size_t)M);
+        else if (V)
+            for (int64_t k = 0; k < M; ++k) V[inv[k]] = v[k];
+        if (ref && same) std::memcpy(ref, r, (size_t)M);
+        else if (ref)
+            for (int64_t k = 0; k < M; ++k) ref[inv[k]] = r[k];
+        if (t) *t = ((const Ctrl *)s->back)->t;
+        return SNN_OK;
+    }
     CK(cudaStreamSynchronize(s->stream));
-    if (V) {
+    if (V && same) {
+        CK(cudaMemcpy(V, s->dev.V, sizeof(float) * (size_t)M, cudaMemcpyDeviceToHost));
+    } else if (V) {
         std::vector<float> b((size_t)M);
         CK(cudaMemcpy(b.data(), s->dev.V, sizeof(float) * (size_t)M, cudaMemcpyDeviceToHost));
         for (int64_t k = 0; k < M; ++k) V[inv[k]] = b[k];
     }
-    if (ref) {
+    if (ref && same) {
+        CK(cudaMemcpy(ref, s->dev.ref, (size_t)M, cudaMemcpyDeviceToHost));
+    } else if (ref) {
         std::vector<uint8_t> b((size_t)M);
         CK(cudaMemcpy(b.data(), s->dev.ref, (size_t)M, cudaMemcpyDeviceToHost));
         for (int64_t k = 0; k < M; ++k) ref[inv[k]] = b[k];

@@ -2,54 +2,77 @@
 // growth, the parallel form of the greedy that the paper leaves as future
 // work (Sec. VII, parallelization of algorithms).
 //
-// One cooperative launch per iteration t grows parts 0..P-2 one after the
-// other; the last part takes the rest; the host keeps the iteration with the
-// smallest objective.  A part grows in rounds:
+// A cooperative launch runs two iterations t side by side, each on one half of
+// the blocks with its own state and barrier; iteration t grows parts 0..P-2
+// one after the other, the last part takes the rest; the host keeps the
+// iteration with the smallest objective.  A part grows in rounds:
 //   scatter  the members that joined in the last round add their weight W_a
 //            to acc[j] of every neuron j they share a synapse with (either
 //            direction, with multiplicity): gain(j) = W_j * acc[j] is
 //            sum_{i in part} (c_ij + c_ji) W_i W_j;
-//   select   the `need` unassigned neurons with the largest gains (ties:
-//            lowest id) by a radix select over unique 64-bit keys
-//            (gain << idbits | (2^idbits - 1 - j)), 11 bits per pass, one
-//            shared-memory histogram per block merged into a global one;
-//   join     block 0 sorts the round's members by key and lets them join in
-//            that order until the part's weight reaches sum(W)/P.
+//   select   a histogram of the unassigned neurons' gains on a logarithmic
+//            scale gives a bound that the `need` largest unique 64-bit keys
+//            (gain << idbits | (2^idbits - 1 - j): ties to the lowest id) all
+//            reach and at most kMaxBatch keys do (further histograms split
+//            the bound's bin while more do); those keys are listed;
+//   join     every block sorts the listed keys by itself, and the first
+//            `need` join in that order until the part's weight reaches
+//            sum(W)/P: each block keeps the labels of its own neurons and
+//            the part's size and weight, so nothing is sent after the join.
 // need = min(B, unassigned, max(1, n_k / g)) (g = 0 drops the last term),
 // n_k = the part's size so far.  Every step is integer arithmetic, so the
 // result does not depend on the order of the atomic additions: it equals the
 // sequential reading with the same rounds bit for bit, and with B = 1 the
 // one-neuron-at-a-time greedy.  Grid barriers are bounded (a block that
 // waits past the limit records a timeout and the launch ends).
+//
+// The rounds are short (65,536 neurons of 200 synapses into 16 parts: 1,260
+// rounds over 4 iterations), so what bounds them is the chain of barriers and
+// of steps between them, not the memory.  Hence three barriers per round
+// (after the scatter, the histogram and the listing), one block per SM, and
+// two iterations at once.  Building that network up to its first 100 steps
+// (lists, this partition, routing tables, sim) takes 25 ms; 68 with seven
+// barriers per round (four histogram passes over the keys, the join on one
+// block), two blocks per SM and one iteration at a time.
 #include <cuda_runtime.h>
 
 #include "snn_internal.h"
 
 namespace {
 
-constexpr int kPT = 256;                 // threads per block
+constexpr int kPT = 1024;                // threads per block
 constexpr int kPW = kPT / 32;
-constexpr int kDigit = 11;               // radix digit bits
+constexpr int kDigit = 11;               // digit bits of the histograms
 constexpr int kBins = 1 << kDigit;
-constexpr int kMaxPass = (64 + kDigit - 1) / kDigit;
+constexpr int kHists = 3;                // global histograms in turn: filled, read, cleared
+constexpr int kGroups = 2;               // iterations side by side
 constexpr int kMaxBatch = 2048;          // largest round
 constexpr int kChunk = 256;              // synapses per scatter task
+constexpr int kPUnroll = kChunk / 32;    // loads in flight per lane
 
 constexpr uint32_t kPStTimeout = 1u, kPStRange = 2u, kPStFault = 4u;
 
 struct PCtl {
-    alignas(128) unsigned long long bar;  // grid-barrier arrivals of the running launch
-    alignas(128) unsigned int nsel;       // members found by the selection
+    alignas(128) unsigned long long bar;  // barrier arrivals of the running launch
+    alignas(128) unsigned int nsel;       // keys listed by the selection
     alignas(128) unsigned int status;
-    unsigned int seed_id;                 // seed of part k: lowest unassigned id (t == 1, atomicMin) or the
-                                          // drawn one (t > 1); all ones between parts
-    int stop;                             // part k is full
-    int na;                               // members that joined in the last round
-    long long wk, nk, n_un;               // weight and size of part k, unassigned neurons
+    unsigned int seed_id[3];              // seed of part k at k % 3: lowest unassigned id (t == 1, atomicMin) or
+                                          // the drawn one (t > 1); all ones until then
     unsigned long long obj;               // objective of the iteration
-    // setup results
+    // setup results (group 0)
     unsigned long long gain_max;          // largest possible gain
     unsigned long long deg_max;           // largest out- or in-degree
+};
+
+// State of one iteration.
+struct PGroup {
+    unsigned long long *acc;    // [M] weight shared with the growing part
+    int32_t *lab;               // [M] part of each neuron (-1: unassigned)
+    uint32_t *hist;             // [kHists][kBins]
+    unsigned long long *sel;    // [kMaxBatch] keys listed by the selection
+    uint32_t *cnt;              // [blocks] unassigned neurons per block
+    unsigned long long *wpart;  // [P] part weights
+    PCtl *c;
 };
 
 struct PDev {
@@ -58,19 +81,12 @@ struct PDev {
     long long *in_ptr;          // [M+1] in-synapses of each neuron
     uint32_t *in_src;           // [E]
     uint32_t *W;                // [M] out-degree
-    unsigned long long *acc;    // [M] weight shared with the growing part
-    unsigned long long *key;    // [M] selection key of the round (0: assigned)
-    int32_t *lab;               // [M] part of each neuron (-1: unassigned)
     uint32_t *fill;             // [M] in-degree counters of the in-list build
-    uint32_t *hist;             // [2][kMaxPass][kBins] by round parity
-    unsigned long long *sel;    // [kMaxBatch] keys of the round's members
-    uint32_t *added;            // [kMaxBatch] members that joined in the last round
-    uint32_t *cnt;              // [grid] unassigned neurons per block
-    const uint32_t *rword;      // [P] Philox words of the seeds (t > 1)
-    unsigned long long *wpart;  // [P] part weights of the iteration
-    PCtl *c;
+    PGroup g[kGroups];
     long long M, E, Wtot;
-    int P, B, grow, t, idbits, nbits, npass, chunks;
+    int P, B, grow, idbits, mbits, chunks;
+    int t0, groups, blocks;     // the launch runs iterations t0 .. t0 + groups - 1 on `blocks` blocks each
+    uint64_t seed;
     unsigned long long limit_ns;
 };
 
@@ -81,18 +97,18 @@ __device__ __forceinline__ unsigned long long p_ns()
     return t;
 }
 
-// Bounded grid barrier number k of the launch (cooperative: every block is
-// resident).  A block-wide barrier, a release add and acquire loads at GPU
+// Bounded barrier number k of an iteration's blocks (cooperative launch: every
+// block is resident).  A block-wide barrier, a release add and acquire loads at GPU
 // scope make the writes of every block before it visible after it.  Returns
 // false (after recording kPStTimeout) when the wait runs out or another
 // block's did.
-__device__ __forceinline__ bool p_sync(PCtl *c, unsigned long long k, unsigned long long limit_ns)
+__device__ __forceinline__ bool p_sync(PCtl *c, unsigned long long k, int blocks, unsigned long long limit_ns)
 {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        const unsigned long long target = (k + 1ull) * gridDim.x;
+        const unsigned long long target = (k + 1ull) * (unsigned long long)blocks;
         asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&c->bar) : "memory");
         const unsigned long long deadline = p_ns() + limit_ns;
         unsigned int spins = 0;
@@ -100,7 +116,7 @@ __device__ __forceinline__ bool p_sync(PCtl *c, unsigned long long k, unsigned l
             unsigned long long v;
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&c->bar) : "memory");
             if (v >= target) break;
-            if ((++spins & 15u) == 0u) {
+            if ((++spins & 63u) == 0u) {
                 if (*(volatile unsigned int *)&c->status & kPStTimeout) {
                     ok = 0;
                     break;
@@ -111,7 +127,6 @@ __device__ __forceinline__ bool p_sync(PCtl *c, unsigned long long k, unsigned l
                     break;
                 }
             }
-            __nanosleep(32);
         }
         s_ok = ok;
     }
@@ -167,7 +182,7 @@ __global__ void k_part_degrees(PDev d)
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < d.E; e += stride) {
         const uint32_t j = d.tgt[e];
         if (j < (unsigned long long)d.M) atomicAdd(&d.fill[j], 1u);
-        else atomicOr(&d.c->status, kPStRange);
+        else atomicOr(&d.g[0].c->status, kPStRange);
     }
 }
 
@@ -236,338 +251,367 @@ __global__ void k_part_bounds(PDev d)
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         if (lane == 0) {
             const unsigned long long wj = d.W[j];
-            if (__umul64hi(wj, s) != 0ull) atomicOr(&d.c->status, kPStRange);
-            atomicMax(&d.c->gain_max, wj * s);
+            if (__umul64hi(wj, s) != 0ull) atomicOr(&d.g[0].c->status, kPStRange);
+            atomicMax(&d.g[0].c->gain_max, wj * s);
             const unsigned long long dg = max(d.ptr[j + 1] - d.ptr[j], d.in_ptr[j + 1] - d.in_ptr[j]);
-            atomicMax(&d.c->deg_max, dg);
+            atomicMax(&d.g[0].c->deg_max, dg);
         }
     }
 }
 
 // ------------------------------------------------------------------ growth
-struct PShared {
-    union {
-        uint32_t hist[kBins];
-        struct {
-            unsigned long long key[kMaxBatch];
-            long long pre[kMaxBatch];
-        } s;
-    } u;
-    long long red64[kPW];
-    unsigned long long redu[kPW];
-    uint32_t red32[kPW];
-    long long n_un, nk, wk;
-    int stop, na, digit;
-    unsigned long long above;
-    unsigned int seed;
-};
-
-// Neuron slice [lo, hi) of this block.
-__device__ __forceinline__ void p_slice(const PDev &d, long long &lo, long long &hi)
+// Word 0 of Philox4x32-10 at counter (c0, c1, c2, 0).
+__device__ __noinline__ uint32_t p_philox_word0(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2)
 {
-    lo = d.M * blockIdx.x / gridDim.x;
-    hi = d.M * (blockIdx.x + 1) / gridDim.x;
+    uint32_t x[4] = {c0, c1, c2, 0u};
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    for (int r = 0; r < 10; ++r) {
+        const uint32_t h0 = __umulhi(0xD2511F53u, x[0]), l0 = 0xD2511F53u * x[0];
+        const uint32_t h1 = __umulhi(0xCD9E8D57u, x[2]), l1 = 0xCD9E8D57u * x[2];
+        x[0] = h1 ^ x[1] ^ k0;
+        x[1] = l1;
+        x[2] = h0 ^ x[3] ^ k1;
+        x[3] = l0;
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return x[0];
 }
 
-// Thread 0 reads the control words written before the last barrier.
-__device__ __forceinline__ void p_read_ctl(const PDev &d, PShared &sh)
+struct PShared {
+    uint32_t hist[kBins];
+    unsigned long long key[kMaxBatch];  // listed keys, then sorted
+    uint32_t added[kMaxBatch];          // members that joined in the last round
+    uint32_t cut;                       // bin of the need-th largest key, keys in the bins above it, in it
+    uint32_t above, in;
+    uint32_t n, base, seed;
+    unsigned long long redu[kPW];
+    uint32_t red32[kPW];
+};
+
+// Bin of a gain: exact below 2^mb, then 2^mb bins per power of two (an
+// increasing function); p_bin_range inverts it to a range of keys.
+__device__ __forceinline__ uint32_t p_bin(unsigned long long gain, int mb)
 {
-    if (threadIdx.x == 0) {
-        volatile PCtl *c = d.c;
-        sh.n_un = c->n_un;
-        sh.nk = c->nk;
-        sh.wk = c->wk;
-        sh.stop = c->stop;
-        sh.na = c->na;
+    if (gain < (1ull << mb)) return (uint32_t)gain;
+    const int e = 63 - __clzll((long long)gain);
+    return ((uint32_t)(e - mb) << mb) + (uint32_t)(gain >> (e - mb));
+}
+__device__ __forceinline__ void p_bin_range(uint32_t bin, int mb, int idbits, unsigned long long &base, int &width)
+{
+    // (bins e << mb | m of e >= 1 stand for gains (2^mb + m) << (e - 1))
+    const int e = (int)(bin >> mb);
+    const unsigned long long m = bin & ((1u << mb) - 1u);
+    const int sh = max(0, e - 1);
+    base = ((e ? m + (1ull << mb) : m) << sh) << idbits;
+    width = sh + idbits;
+}
+
+// Adds the block's histogram to the global one h, clears `next` (this block's
+// share), passes the barrier and finds the bin of the need-th largest key.
+__device__ __forceinline__ bool p_cut(const PDev &d, const PGroup &g, PShared &sh, int rank, uint32_t *h,
+                                      uint32_t *next, uint32_t need, unsigned long long &bk)
+{
+    __syncthreads();
+    for (int x = threadIdx.x; x < kBins; x += kPT)
+        if (sh.hist[x]) atomicAdd(h + x, sh.hist[x]);
+    for (int x = rank * kPT + threadIdx.x; x < kBins; x += d.blocks * kPT) next[x] = 0u;
+    if (!p_sync(g.c, bk++, d.blocks, d.limit_ns)) return false;
+    constexpr int kPer = kBins / kPT;
+    uint32_t v[kPer], s = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        v[q] = __ldcg(h + threadIdx.x * kPer + q);
+        s += v[q];
     }
+    uint32_t tot;
+    const uint32_t ex = p_block_excl(s, sh.red32, tot);
+    uint32_t above = tot - ex - s;  // keys in the bins above this thread's
+#pragma unroll
+    for (int q = kPer - 1; q >= 0; --q) {
+        if (above < need && above + v[q] >= need) {
+            sh.cut = (uint32_t)(threadIdx.x * kPer + q);
+            sh.above = above;
+            sh.in = v[q];
+        }
+        above += v[q];
+    }
+    __syncthreads();
+    return true;
+}
+
+// Sorts key[0 .. n2), n2 a power of two >= 64, in decreasing order.  A warp
+// holds the pairs of 64 keys in a row, so strides up to 32 need no block
+// barrier.
+__device__ __forceinline__ void p_sort(unsigned long long *key, int n2)
+{
+    static_assert(kMaxBatch <= 2 * kPT, "one pair per thread");
+    const int x = threadIdx.x;
+    const bool mine = x < (n2 >> 1);
+    for (int size = 2; size <= n2; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            if (stride > 32 || (stride == 32 && size > 64)) __syncthreads();
+            else __syncwarp();
+            if (mine) {
+                const int i = ((x & ~(stride - 1)) << 1) | (x & (stride - 1)), j = i + stride;
+                const unsigned long long a = key[i], b = key[j];
+                if ((i & size) == 0 ? a < b : a > b) {
+                    key[i] = b;
+                    key[j] = a;
+                }
+            }
+        }
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kPT) k_part_grow(PDev d)
+__global__ void __launch_bounds__(kPT, 1) k_part_grow(const PDev d)
 {
     __shared__ PShared sh;
-    PCtl *c = d.c;
-    long long lo, hi;
-    p_slice(d, lo, hi);
-    unsigned long long bk = 0;  // barriers passed
-    unsigned int round = 0;
+    const int grp = blockIdx.x / d.blocks, rank = blockIdx.x - grp * d.blocks, t = d.t0 + grp;
+    const PGroup g = d.g[grp];
+    PCtl *c = g.c;
+    // this block's neurons
+    const long long lo = d.M * rank / d.blocks, hi = d.M * (rank + 1) / d.blocks;
+    const int lane = threadIdx.x & 31, tid = threadIdx.x;
+    const long long gwarp = ((long long)rank * kPT + tid) >> 5, nwarp = ((long long)d.blocks * kPT) >> 5;
     const unsigned long long idmask = (1ull << d.idbits) - 1ull;
-    const int lane = threadIdx.x & 31;
-    const long long gwarp = ((long long)blockIdx.x * kPT + threadIdx.x) >> 5;
-    const long long nwarp = ((long long)gridDim.x * kPT) >> 5;
+    unsigned long long bk = 0;  // barriers passed
+    int hcur = 0;               // histogram to fill next
+    long long n_un = d.M;       // unassigned neurons (the same in every block, as all of the part's state)
     bool ok = true;
 
-    for (int k = 0; k < d.P - 1 && ok; ++k) {
-        p_read_ctl(d, sh);
-        if (sh.n_un == 0) break;
+    for (int k = 0; k < d.P - 1 && ok && n_un > 0; ++k) {
         // a new part: clear the shared weights; find the seed
-        for (long long j = lo + threadIdx.x; j < hi; j += kPT) d.acc[j] = 0ull;
-        if (d.t == 1) {
-            unsigned int m = 0xFFFFFFFFu;
-            for (long long j = lo + threadIdx.x; j < hi; j += kPT)
-                if (__ldcg(d.lab + j) < 0) {
-                    m = (unsigned int)j;
-                    break;
-                }
-            m = __reduce_min_sync(0xFFFFFFFFu, m);
-            if (lane == 0) sh.red32[threadIdx.x >> 5] = m;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned int b = 0xFFFFFFFFu;
-                for (int w = 0; w < kPW; ++w) b = min(b, sh.red32[w]);
-                if (b != 0xFFFFFFFFu) atomicMin(&c->seed_id, b);
+        unsigned int m = 0xFFFFFFFFu, n = 0;
+        for (long long j = lo + tid; j < hi; j += kPT) {
+            g.acc[j] = 0ull;
+            if (__ldcg(g.lab + j) < 0) {
+                ++n;
+                m = min(m, (unsigned int)j);
             }
-        } else {
-            unsigned int n = 0;
-            for (long long j = lo + threadIdx.x; j < hi; j += kPT) n += __ldcg(d.lab + j) < 0;
-            n = p_block_sum(n, sh.red32);
-            if (threadIdx.x == 0) d.cnt[blockIdx.x] = n;
         }
-        if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
-        if (d.t != 1) {
+        unsigned int *seed_id = &c->seed_id[k % 3];
+        if (t == 1) {
+            m = __reduce_min_sync(0xFFFFFFFFu, m);
+            if (lane == 0 && m != 0xFFFFFFFFu) atomicMin(seed_id, m);
+        } else {
+            n = p_block_sum(n, sh.red32);
+            if (tid == 0) g.cnt[rank] = n;
+        }
+        if (!(ok = p_sync(c, bk++, d.blocks, d.limit_ns))) break;
+        if (t != 1) {
             // the r-th unassigned neuron in id order, r = word mod unassigned
-            const unsigned long long r = (unsigned long long)d.rword[k] % (unsigned long long)sh.n_un;
+            const unsigned long long r =
+                (unsigned long long)p_philox_word0(d.seed, (uint32_t)t, (uint32_t)k, 0xA1u) % (unsigned long long)n_un;
             unsigned long long pre = 0;
-            for (int x = threadIdx.x; x < (int)blockIdx.x; x += kPT) pre += __ldcg(d.cnt + x);
+            for (int x = tid; x < rank; x += kPT) pre += __ldcg(g.cnt + x);
             pre = p_block_sum(pre, sh.redu);
-            const unsigned long long mine = __ldcg(d.cnt + blockIdx.x);
+            const unsigned long long mine = __ldcg(g.cnt + rank);
             if (r >= pre && r < pre + mine) {
                 // walk the slice in blocks of kPT ids, scanning the flags
-                unsigned long long need = r - pre;
+                unsigned long long want = r - pre;
                 for (long long j0 = lo; j0 < hi; j0 += kPT) {
-                    const long long j = j0 + threadIdx.x;
-                    const unsigned int f = (j < hi && __ldcg(d.lab + j) < 0) ? 1u : 0u;
+                    const long long j = j0 + tid;
+                    const unsigned int f = (j < hi && __ldcg(g.lab + j) < 0) ? 1u : 0u;
                     unsigned int tot;
                     const unsigned int ex = p_block_excl(f, sh.red32, tot);
-                    if (f && ex == need) c->seed_id = (unsigned int)j;
-                    if (need < tot) break;
-                    need -= tot;
+                    if (f && ex == want) *(volatile unsigned int *)seed_id = (unsigned int)j;
+                    if (want < tot) break;
+                    want -= tot;
                 }
             }
-            if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
+            if (!(ok = p_sync(c, bk++, d.blocks, d.limit_ns))) break;
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            const unsigned int s = *(volatile unsigned int *)&c->seed_id;
-            c->seed_id = 0xFFFFFFFFu;
-            if (s >= (unsigned long long)d.M) {
-                // no seed found: record it and end the growth
-                atomicOr(&c->status, kPStFault);
-                c->stop = 1;
-                c->n_un = 0;
-            } else {
-            d.lab[s] = k;
-            d.added[0] = s;
-            const long long wk = d.W[s];
-            const long long n_un = sh.n_un - 1;
-            c->wk = wk;
-            c->nk = 1;
-            c->n_un = n_un;
-            c->na = 1;
-            c->stop = !(wk * (long long)d.P < d.Wtot) || n_un == 0;
-            }
+        const unsigned int seed = __ldcg(seed_id);
+        // (the word of part k + 2: last read before this part's first barrier)
+        if (rank == 0 && tid == 0) *(volatile unsigned int *)&c->seed_id[(k + 2) % 3] = 0xFFFFFFFFu;
+        if (seed >= (unsigned long long)d.M) {
+            // no seed found (the same in every block): record it and end
+            if (tid == 0) atomicOr(&c->status, kPStFault);
+            return;
         }
-        if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
+        if (tid == 0) {
+            sh.added[0] = seed;
+            if (seed >= lo && seed < hi) g.lab[seed] = k;
+        }
+        __syncthreads();
+        long long wk = d.W[seed], nk = 1;  // weight and size of part k
+        int na = 1;                        // members that joined in the last round
+        --n_un;
 
-        for (;;) {
-            p_read_ctl(d, sh);
-            if (sh.stop) break;
-            const int par = (int)(round & 1u);
-            ++round;
+        while (wk * (long long)d.P < d.Wtot && n_un > 0) {
             // scatter: (member, direction, chunk of kChunk synapses) per warp
-            const long long tasks = (long long)sh.na * 2 * d.chunks;
+            const long long tasks = (long long)na * 2 * d.chunks;
             for (long long x = gwarp; x < tasks; x += nwarp) {
-                const uint32_t a = __ldcg(d.added + x / (2 * d.chunks));
-                const int rem = (int)(x % (2 * d.chunks));
+                const long long mem = x / (2 * d.chunks);
+                const uint32_t a = sh.added[mem];
+                const int rem = (int)(x - mem * (2 * d.chunks));
                 const bool in = rem >= d.chunks;
                 const long long ch = rem - (in ? d.chunks : 0);
-                const long long b0 = in ? d.in_ptr[a] : d.ptr[a];
-                const long long b1 = in ? d.in_ptr[a + 1] : d.ptr[a + 1];
-                const long long s0 = b0 + ch * kChunk;
-                const long long s1 = min(b1, s0 + kChunk);
+                const long long *ptr = in ? d.in_ptr : d.ptr;
+                const uint32_t *list = in ? d.in_src : d.tgt;
+                const long long s0 = ptr[a] + ch * kChunk, s1 = min(ptr[a + 1], s0 + kChunk);
                 const unsigned long long wa = d.W[a];
-                for (long long e = s0 + lane; e < s1; e += 32) {
-                    const uint32_t j = in ? d.in_src[e] : d.tgt[e];
-                    atomicAdd(d.acc + j, wa);
-                }
+                uint32_t j[kPUnroll];
+#pragma unroll
+                for (int q = 0; q < kPUnroll; ++q)
+                    if (s0 + lane + 32 * q < s1) j[q] = list[s0 + lane + 32 * q];
+#pragma unroll
+                for (int q = 0; q < kPUnroll; ++q)
+                    if (s0 + lane + 32 * q < s1) atomicAdd(g.acc + j[q], wa);
             }
-            long long need = min((long long)d.B, sh.n_un);
-            if (d.grow > 0) need = min(need, max(1ll, sh.nk / d.grow));
-            if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
+            uint32_t need = (uint32_t)min((long long)d.B, n_un);
+            if (d.grow > 0) need = (uint32_t)min((long long)need, max(1ll, nk / d.grow));
+            for (int x = tid; x < kBins; x += kPT) sh.hist[x] = 0u;
+            if (!(ok = p_sync(c, bk++, d.blocks, d.limit_ns))) break;
+            if (rank == 0 && tid == 0) *(volatile unsigned int *)&c->nsel = 0u;
 
-            // select: the need-th largest key by radix passes over the digits
-            uint32_t *gh = d.hist + (size_t)par * kMaxPass * kBins;
-            unsigned long long prefix = 0, mask = 0;
-            unsigned long long remk = (unsigned long long)need;
-            for (int p = 0; p < d.npass && ok; ++p) {
-                const int top = d.nbits - kDigit * p;
-                const int shift = max(0, top - kDigit);
-                const unsigned long long dmask = (1ull << (top - shift)) - 1ull;
-                for (int x = threadIdx.x; x < kBins; x += kPT) sh.u.hist[x] = 0u;
+            // select: bins of the gains; neurons without gain count per warp
+            const auto key_of = [&](long long j) -> unsigned long long {
+                return __ldcg(g.lab + j) >= 0 ? 0ull
+                                              : (unsigned long long)d.W[j] * __ldcg(g.acc + j) << d.idbits |
+                                                    (idmask - (unsigned long long)j);
+            };
+            for (long long j0 = lo; j0 < hi; j0 += kPT) {
+                const long long j = j0 + tid;
+                const unsigned long long kj = j < hi ? key_of(j) : 0ull;
+                const uint32_t bin = p_bin(kj >> d.idbits, d.mbits);
+                const unsigned int zero = __ballot_sync(0xFFFFFFFFu, kj != 0ull && bin == 0u);
+                if (kj != 0ull && bin != 0u) atomicAdd(&sh.hist[bin], 1u);
+                if (lane == 0 && zero) atomicAdd(&sh.hist[0], (uint32_t)__popc(zero));
+            }
+            int hnext = hcur == kHists - 1 ? 0 : hcur + 1;
+            if (!(ok = p_cut(d, g, sh, rank, g.hist + hcur * kBins, g.hist + hnext * kBins, need, bk))) break;
+            hcur = hnext;
+            unsigned long long base;  // the bound's bin: keys base .. base + 2^width - 1
+            int width;
+            p_bin_range(sh.cut, d.mbits, d.idbits, base, width);
+            uint32_t above = sh.above, in = sh.in;
+            while (above + in > (uint32_t)kMaxBatch && width > 0) {
+                // more keys reach the bin than a round's list holds: split it
+                const int shift = max(0, width - kDigit);
                 __syncthreads();
-                for (long long j = lo + threadIdx.x; j < hi; j += kPT) {
-                    unsigned long long kj;
-                    if (p == 0) {
-                        kj = 0ull;
-                        if (__ldcg(d.lab + j) < 0)
-                            kj = ((unsigned long long)d.W[j] * __ldcg(d.acc + j)) << d.idbits |
-                                 (idmask - (unsigned long long)j);
-                        d.key[j] = kj;
-                    } else {
-                        kj = d.key[j];
-                    }
-                    if (kj != 0ull && (kj & mask) == prefix) atomicAdd(&sh.u.hist[(kj >> shift) & dmask], 1u);
+                for (int x = tid; x < kBins; x += kPT) sh.hist[x] = 0u;
+                __syncthreads();
+                for (long long j = lo + tid; j < hi; j += kPT) {
+                    const unsigned long long off = key_of(j) - base;
+                    // (an assigned neuron's key 0 lies below every bin's keys but those of base 0, where key 0
+                    // is excluded by itself)
+                    if (off >> width == 0ull && off + base != 0ull) atomicAdd(&sh.hist[off >> shift], 1u);
                 }
-                __syncthreads();
-                for (int x = threadIdx.x; x < kBins; x += kPT)
-                    if (sh.u.hist[x]) atomicAdd(gh + p * kBins + x, sh.u.hist[x]);
-                if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
-                // the digit whose bin holds the remk-th largest key
-                constexpr int kPer = kBins / kPT;
-                uint32_t v[kPer];
-                unsigned long long s = 0;
-#pragma unroll
-                for (int q = 0; q < kPer; ++q) {
-                    v[q] = __ldcg(gh + p * kBins + threadIdx.x * kPer + q);
-                    s += v[q];
-                }
-                // suffix sums over threads: keys in bins above this thread's
-                unsigned long long tot;
-                const unsigned long long ex = p_block_excl(s, sh.redu, tot);
-                unsigned long long above = tot - ex - s;
-#pragma unroll
-                for (int q = kPer - 1; q >= 0; --q) {
-                    if (above < remk && above + v[q] >= remk) {
-                        sh.digit = threadIdx.x * kPer + q;
-                        sh.above = above;
-                    }
-                    above += v[q];
-                }
-                __syncthreads();
-                remk -= sh.above;
-                prefix |= (unsigned long long)sh.digit << shift;
-                mask |= dmask << shift;
-                __syncthreads();
+                hnext = hcur == kHists - 1 ? 0 : hcur + 1;
+                if (!(ok = p_cut(d, g, sh, rank, g.hist + hcur * kBins, g.hist + hnext * kBins, need - above, bk)))
+                    break;
+                hcur = hnext;
+                base += (unsigned long long)sh.cut << shift;
+                width = shift;
+                above += sh.above;
+                in = sh.in;
             }
             if (!ok) break;
-            // the keys are unique: the need members are the keys >= prefix
-            {
-                uint32_t *other = d.hist + (size_t)(par ^ 1) * kMaxPass * kBins;
-                for (long long x = (long long)blockIdx.x * kPT + threadIdx.x; x < kMaxPass * kBins;
-                     x += (long long)gridDim.x * kPT)
-                    other[x] = 0u;
-            }
-            for (long long j = lo + threadIdx.x; j < hi; j += kPT) {
-                const unsigned long long kj = d.key[j];
-                if (kj != 0ull && kj >= prefix) {
-                    const unsigned int pos = atomicAdd(&c->nsel, 1u);
-                    if (pos < (unsigned int)kMaxBatch) d.sel[pos] = kj;  // (more is a fault, flagged below)
+            const uint32_t ns = above + in;
+            // list the keys >= base: this block's into shared memory, then one place in the list for them
+            if (tid == 0) sh.n = 0u;
+            __syncthreads();
+            for (long long j = lo + tid; j < hi; j += kPT) {
+                const unsigned long long kj = key_of(j);
+                if (kj != 0ull && kj >= base) {
+                    const uint32_t pos = atomicAdd(&sh.n, 1u);
+                    if (pos < (uint32_t)kMaxBatch) sh.key[pos] = kj;  // (more is a fault, flagged below)
                 }
             }
-            if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
+            __syncthreads();
+            if (tid == 0 && sh.n) sh.base = atomicAdd(&c->nsel, sh.n);
+            __syncthreads();
+            for (uint32_t x = tid; x < min(sh.n, (uint32_t)kMaxBatch); x += kPT)
+                if (sh.base + x < (uint32_t)kMaxBatch) g.sel[sh.base + x] = sh.key[x];
+            if (!(ok = p_sync(c, bk++, d.blocks, d.limit_ns))) break;
 
-            // join (block 0): sort the members by key, descending; they join
-            // in that order while the part's weight is below sum(W)/P
-            if (blockIdx.x == 0) {
-                const unsigned int nsel = *(volatile unsigned int *)&c->nsel;
-                if (nsel != (unsigned int)need) {
-                    // not the round's size: record it and end the growth
-                    if (threadIdx.x == 0) {
-                        atomicOr(&c->status, kPStFault);
-                        c->stop = 1;
-                        c->n_un = 0;
-                        c->nsel = 0u;
-                    }
-                    goto joined;
-                }
-                const int n = (int)nsel;
-                int n2 = 1;
-                while (n2 < n) n2 <<= 1;
-                for (int x = threadIdx.x; x < n2; x += kPT) sh.u.s.key[x] = x < n ? __ldcg(d.sel + x) : 0ull;
-                __syncthreads();
-                for (int size = 2; size <= n2; size <<= 1)
-                    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                        for (int x = threadIdx.x; x < n2; x += kPT) {
-                            const int y = x ^ stride;
-                            if (y > x) {
-                                const bool desc = (x & size) == 0;
-                                const unsigned long long a = sh.u.s.key[x], b = sh.u.s.key[y];
-                                if (desc ? a < b : a > b) {
-                                    sh.u.s.key[x] = b;
-                                    sh.u.s.key[y] = a;
-                                }
-                            }
-                        }
-                        __syncthreads();
-                    }
-                // inclusive prefix sums of the members' weights, kPer per thread
-                constexpr int kPer = kMaxBatch / kPT;
-                long long w[kPer];
-                long long s = 0;
-#pragma unroll
-                for (int q = 0; q < kPer; ++q) {
-                    const int x = threadIdx.x * kPer + q;
-                    w[q] = x < n ? (long long)d.W[idmask - (sh.u.s.key[x] & idmask)] : 0ll;
-                    s += w[q];
-                }
-                long long tot;
-                long long run = p_block_excl(s, sh.red64, tot);
-#pragma unroll
-                for (int q = 0; q < kPer; ++q) {
-                    run += w[q];
-                    const int x = threadIdx.x * kPer + q;
-                    if (x < n) sh.u.s.pre[x] = run;
-                }
-                __syncthreads();
-                // members before the first one whose join fills the part
-                unsigned int cont = 0;
-                for (int x = threadIdx.x; x < n; x += kPT)
-                    cont += ((sh.wk + sh.u.s.pre[x]) * (long long)d.P < d.Wtot) && (sh.n_un - x - 1 > 0);
-                const int m = min(n, (int)p_block_sum(cont, sh.red32) + 1);
-                for (int x = threadIdx.x; x < m; x += kPT) {
-                    const uint32_t id = (uint32_t)(idmask - (sh.u.s.key[x] & idmask));
-                    d.lab[id] = k;
-                    d.added[x] = id;
-                }
-                if (threadIdx.x == 0) {
-                    const long long wk = sh.wk + sh.u.s.pre[m - 1];
-                    const long long n_un = sh.n_un - m;
-                    c->wk = wk;
-                    c->nk = sh.nk + m;
-                    c->n_un = n_un;
-                    c->na = m;
-                    c->stop = !(wk * (long long)d.P < d.Wtot) || n_un == 0;
-                    c->nsel = 0u;
-                }
+            // join: the listed keys in decreasing order; the first `need`
+            // join while the part's weight is below sum(W)/P
+            if (__ldcg(&c->nsel) != ns || ns < need || ns > (uint32_t)kMaxBatch) {
+                // not the round's size (the same in every block): record it and end
+                if (tid == 0) atomicOr(&c->status, kPStFault);
+                return;
             }
-        joined:
-            if (!(ok = p_sync(c, bk++, d.limit_ns))) break;
+            int n2 = 64;
+            while (n2 < (int)ns) n2 <<= 1;
+            for (int x = tid; x < n2; x += kPT) sh.key[x] = x < (int)ns ? __ldcg(g.sel + x) : 0ull;
+            __syncthreads();
+            p_sort(sh.key, n2);
+            // inclusive prefix sums of the members' weights, kPer per thread
+            constexpr int kPer = kMaxBatch / kPT;
+            long long w[kPer], s = 0;
+            uint32_t id[kPer];
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                const int x = tid * kPer + q;
+                w[q] = 0;
+                if (x < (int)need) {
+                    id[q] = (uint32_t)(idmask - (sh.key[x] & idmask));
+                    w[q] = (long long)d.W[id[q]];
+                }
+                s += w[q];
+            }
+            unsigned long long tot;
+            long long run = (long long)p_block_excl((unsigned long long)s, sh.redu, tot);
+            // members before the first one whose join fills the part
+            unsigned int cont = 0;
+            long long pre[kPer];
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                run += w[q];
+                pre[q] = run;
+                const int x = tid * kPer + q;
+                cont += x < (int)need && (wk + run) * (long long)d.P < d.Wtot && n_un - x - 1 > 0;
+            }
+            na = min((int)need, (int)p_block_sum(cont, sh.red32) + 1);
+#pragma unroll
+            for (int q = 0; q < kPer; ++q) {
+                const int x = tid * kPer + q;
+                if (x >= na) continue;
+                sh.added[x] = id[q];
+                if (id[q] >= lo && id[q] < hi) g.lab[id[q]] = k;
+                if (x == na - 1) sh.redu[0] = (unsigned long long)pre[q];
+            }
+            __syncthreads();
+            wk += (long long)sh.redu[0];
+            nk += na;
+            n_un -= na;
         }
     }
     if (!ok) return;
     // the last part takes the rest
-    for (long long j = lo + threadIdx.x; j < hi; j += kPT)
-        if (__ldcg(d.lab + j) < 0) d.lab[j] = d.P - 1;
-    if (!p_sync(c, bk++, d.limit_ns)) return;
+    __syncthreads();
+    for (long long j = lo + tid; j < hi; j += kPT)
+        if (__ldcg(g.lab + j) < 0) g.lab[j] = d.P - 1;
+    if (!p_sync(c, bk++, d.blocks, d.limit_ns)) return;
     // objective (sum over cut synapses of W_i W_j) and part weights; one
     // warp per source neuron
     unsigned long long cut = 0;
     for (long long i = gwarp; i < d.M; i += nwarp) {
-        const int li = __ldcg(d.lab + i);
+        const int li = __ldcg(g.lab + i);
         const unsigned long long wi = d.W[i];
-        if (lane == 0) atomicAdd(d.wpart + li, wi);
-        for (long long e = d.ptr[i] + lane; e < d.ptr[i + 1]; e += 32) {
-            const uint32_t j = d.tgt[e];
-            if (__ldcg(d.lab + j) != li) cut += wi * d.W[j];
+        if (lane == 0) atomicAdd(g.wpart + li, wi);
+        for (long long e0 = d.ptr[i] + lane; e0 < d.ptr[i + 1]; e0 += 32 * kPUnroll) {
+            uint32_t j[kPUnroll];
+            int lj[kPUnroll];
+#pragma unroll
+            for (int q = 0; q < kPUnroll; ++q) j[q] = e0 + 32 * q < d.ptr[i + 1] ? d.tgt[e0 + 32 * q] : (uint32_t)i;
+#pragma unroll
+            for (int q = 0; q < kPUnroll; ++q) lj[q] = __ldcg(g.lab + j[q]);
+#pragma unroll
+            for (int q = 0; q < kPUnroll; ++q)
+                if (lj[q] != li) cut += wi * d.W[j[q]];
         }
     }
     cut = p_block_sum(cut, sh.redu);
-    if (threadIdx.x == 0 && cut) atomicAdd(&c->obj, cut);
+    if (tid == 0 && cut) atomicAdd(&c->obj, cut);
 }
 
 // ------------------------------------------------------------------ host
 struct PLayout {
-    size_t ptr, in_ptr, tgt, in_src, W, acc, key, lab, best, fill, hist, sel, added, cnt, rword, wpart,
-        ctl, total;
+    size_t ctl, ptr, in_ptr, tgt, in_src, W, fill, best, acc[kGroups], lab[kGroups], hist, sel, cnt, wpart, total;
 };
 
 constexpr int kMaxGrid = 4096;
@@ -580,23 +624,22 @@ PLayout p_layout(long long M, long long E, int P)
         f = o;
         o += (bytes + 255) & ~(size_t)255;
     };
-    put(L.ctl, sizeof(PCtl));
+    put(L.ctl, sizeof(PCtl) * kGroups);
     put(L.ptr, 8 * (size_t)(M + 1));
     put(L.in_ptr, 8 * (size_t)(M + 1));
     put(L.tgt, 4 * (size_t)(E > 0 ? E : 1));
     put(L.in_src, 4 * (size_t)(E > 0 ? E : 1));
     put(L.W, 4 * (size_t)M);
-    put(L.acc, 8 * (size_t)M);
-    put(L.key, 8 * (size_t)M);
-    put(L.lab, 4 * (size_t)M);
     put(L.best, 4 * (size_t)M);
-    put(L.fill, 4 * (size_t)M);
-    put(L.hist, 4 * (size_t)2 * kMaxPass * kBins);
-    put(L.sel, 8 * (size_t)kMaxBatch);
-    put(L.added, 4 * (size_t)kMaxBatch);
+    for (int g = 0; g < kGroups; ++g) {
+        put(L.acc[g], 8 * (size_t)M);
+        put(L.lab[g], 4 * (size_t)M);
+    }
+    L.fill = L.lab[0];  // (the in-list build ends before the growth begins)
+    put(L.hist, 4 * (size_t)kGroups * kHists * kBins);
+    put(L.sel, 8 * (size_t)kGroups * kMaxBatch);
     put(L.cnt, 4 * (size_t)kMaxGrid);
-    put(L.rword, 4 * (size_t)P);
-    put(L.wpart, 8 * (size_t)P * 2);
+    put(L.wpart, 8 * (size_t)P * kGroups);
     L.total = o;
     return L;
 }
@@ -659,9 +702,8 @@ extern "C" int snn_partition_device(const snn_network *net, int32_t P, const snn
     if (!coop) return SNN_E_NODEV;
     PCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_part_grow, kPT, 0));
     if (occ < 1) return SNN_E_NODEV;
-    // two blocks per SM: the rounds' barriers cost more with more blocks,
-    // the scatter of a large round wants more than one per SM
-    const int grid = std::min(kMaxGrid, sms * std::min(occ, 2));
+    // one block per SM, shared out among the iterations that run side by side
+    const int grid = std::min(kMaxGrid, sms);
 
     PDev d;
     std::memset(&d, 0, sizeof(d));
@@ -670,29 +712,30 @@ extern "C" int snn_partition_device(const snn_network *net, int32_t P, const snn
     d.in_ptr = (long long *)(w + L.in_ptr);
     d.in_src = (uint32_t *)(w + L.in_src);
     d.W = (uint32_t *)(w + L.W);
-    d.acc = (unsigned long long *)(w + L.acc);
-    d.key = (unsigned long long *)(w + L.key);
-    d.lab = (int32_t *)(w + L.lab);
     d.fill = (uint32_t *)(w + L.fill);
-    d.hist = (uint32_t *)(w + L.hist);
-    d.sel = (unsigned long long *)(w + L.sel);
-    d.added = (uint32_t *)(w + L.added);
-    d.cnt = (uint32_t *)(w + L.cnt);
-    d.rword = (const uint32_t *)(w + L.rword);
-    d.wpart = (unsigned long long *)(w + L.wpart);
-    d.c = (PCtl *)(w + L.ctl);
+    for (int g = 0; g < kGroups; ++g) {
+        PGroup &x = d.g[g];
+        x.acc = (unsigned long long *)(w + L.acc[g]);
+        x.lab = (int32_t *)(w + L.lab[g]);
+        x.hist = (uint32_t *)(w + L.hist) + (size_t)g * kHists * kBins;
+        x.sel = (unsigned long long *)(w + L.sel) + (size_t)g * kMaxBatch;
+        x.cnt = (uint32_t *)(w + L.cnt) + (size_t)g * (kMaxGrid / kGroups);
+        x.wpart = (unsigned long long *)(w + L.wpart) + (size_t)g * P;
+        x.c = (PCtl *)(w + L.ctl) + g;
+    }
     d.M = M;
     d.E = E;
     d.Wtot = E;
     d.P = P;
     d.B = prm->batch;
     d.grow = prm->grow;
+    d.seed = prm->seed;
     d.limit_ns = 2000000000ull;
 
     // tables to the device; in-lists and the key width on the device
     PCK(cudaMemcpyAsync((void *)d.ptr, net->syn_ptr, 8 * (size_t)(M + 1), cudaMemcpyHostToDevice, st));
     if (E > 0) PCK(cudaMemcpyAsync((void *)d.tgt, net->syn_tgt, 4 * (size_t)E, cudaMemcpyHostToDevice, st));
-    PCK(cudaMemsetAsync(d.c, 0, sizeof(PCtl), st));
+    PCK(cudaMemsetAsync(w + L.ctl, 0, sizeof(PCtl), st));
     PCK(cudaMemsetAsync(d.fill, 0, 4 * (size_t)M, st));
     const int g2 = sms * 8;
     k_part_degrees<<<g2, 256, 0, st>>>(d);
@@ -700,44 +743,46 @@ extern "C" int snn_partition_device(const snn_network *net, int32_t P, const snn
     k_part_in_lists<<<g2, 256, 0, st>>>(d);
     k_part_bounds<<<g2, 256, 0, st>>>(d);
     PCK(cudaGetLastError());
-    PCtl ctl;
-    PCK(cudaMemcpyAsync(&ctl, d.c, sizeof(PCtl), cudaMemcpyDeviceToHost, st));
+    PCtl ctl[kGroups];
+    PCK(cudaMemcpyAsync(ctl, w + L.ctl, sizeof(PCtl), cudaMemcpyDeviceToHost, st));
     PCK(cudaStreamSynchronize(st));
-    if (ctl.status & kPStRange) return SNN_E_ARG;
+    if (ctl[0].status & kPStRange) return SNN_E_ARG;
     d.idbits = std::max(1, bit_length((unsigned long long)M));
-    d.nbits = bit_length(ctl.gain_max) + d.idbits;
-    if (d.nbits > 64) return SNN_E_RANGE;
-    d.npass = (d.nbits + kDigit - 1) / kDigit;
-    d.chunks = (int)std::max(1ull, (ctl.deg_max + kChunk - 1) / kChunk);
+    const int gbits = bit_length(ctl[0].gain_max);
+    if (gbits + d.idbits > 64) return SNN_E_RANGE;
+    d.mbits = kDigit;  // as many bins per power of two as the gains' range leaves
+    while ((std::max(0, gbits - d.mbits) + 1) << d.mbits > kBins) --d.mbits;
+    d.chunks = (int)std::max(1ull, (ctl[0].deg_max + kChunk - 1) / kChunk);
 
-    std::vector<uint32_t> rw((size_t)P);
-    unsigned long long best = 0;
-    for (int t = 1; t <= prm->iters; ++t) {
-        for (int k = 0; k < P; ++k) rw[k] = snn::philox_word0(prm->seed, (uint32_t)t, (uint32_t)k, 0xA1u);
-        PCK(cudaMemcpyAsync((void *)d.rword, rw.data(), 4 * (size_t)P, cudaMemcpyHostToDevice, st));
-        std::memset(&ctl, 0, sizeof(ctl));
-        ctl.n_un = M;
-        ctl.seed_id = 0xFFFFFFFFu;
-        PCK(cudaMemcpyAsync(d.c, &ctl, sizeof(PCtl), cudaMemcpyHostToDevice, st));
-        PCK(cudaMemsetAsync(d.lab, 0xFF, 4 * (size_t)M, st));
-        PCK(cudaMemsetAsync(d.hist, 0, 4 * (size_t)2 * kMaxPass * kBins, st));
-        PCK(cudaMemsetAsync(d.wpart, 0, 8 * (size_t)P, st));
-        d.t = t;
-        void *args[] = {&d};
-        PCK(cudaLaunchCooperativeKernel((const void *)k_part_grow, dim3(grid), dim3(kPT), args, 0, st));
-        PCK(cudaMemcpyAsync(&ctl, d.c, sizeof(PCtl), cudaMemcpyDeviceToHost, st));
-        PCK(cudaStreamSynchronize(st));
-        if (ctl.status & kPStTimeout) return SNN_E_TIMEOUT;
-        if (ctl.status & kPStFault) return SNN_E_STATE;
-        if (t == 1 || ctl.obj < best) {
-            best = ctl.obj;
-            PCK(cudaMemcpyAsync(w + L.best, d.lab, 4 * (size_t)M, cudaMemcpyDeviceToDevice, st));
-            PCK(cudaMemcpyAsync(d.wpart + P, d.wpart, 8 * (size_t)P, cudaMemcpyDeviceToDevice, st));
-        }
-    }
     std::vector<unsigned long long> wp((size_t)P);
+    unsigned long long best = 0;
+    for (int t = 1; t <= prm->iters; t += d.groups) {
+        d.t0 = t;
+        d.groups = std::min(kGroups, prm->iters - t + 1);
+        d.blocks = std::max(1, grid / d.groups);
+        std::memset(ctl, 0, sizeof(ctl));
+        for (PCtl &c : ctl)
+            for (unsigned int &x : c.seed_id) x = 0xFFFFFFFFu;
+        PCK(cudaMemcpyAsync(w + L.ctl, ctl, sizeof(ctl), cudaMemcpyHostToDevice, st));
+        for (int g = 0; g < d.groups; ++g) PCK(cudaMemsetAsync(d.g[g].lab, 0xFF, 4 * (size_t)M, st));
+        PCK(cudaMemsetAsync(w + L.hist, 0, 4 * (size_t)kGroups * kHists * kBins, st));
+        PCK(cudaMemsetAsync(w + L.wpart, 0, 8 * (size_t)P * kGroups, st));
+        void *args[] = {&d};
+        PCK(cudaLaunchCooperativeKernel((const void *)k_part_grow, dim3(d.blocks * d.groups), dim3(kPT), args, 0, st));
+        PCK(cudaMemcpyAsync(ctl, w + L.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st));
+        PCK(cudaStreamSynchronize(st));
+        for (int g = 0; g < d.groups; ++g) {
+            if (ctl[g].status & kPStTimeout) return SNN_E_TIMEOUT;
+            if (ctl[g].status & kPStFault) return SNN_E_STATE;
+        }
+        for (int g = 0; g < d.groups; ++g)
+            if (t + g == 1 || ctl[g].obj < best) {
+                best = ctl[g].obj;
+                PCK(cudaMemcpyAsync(w + L.best, d.g[g].lab, 4 * (size_t)M, cudaMemcpyDeviceToDevice, st));
+                PCK(cudaMemcpyAsync(wp.data(), d.g[g].wpart, 8 * (size_t)P, cudaMemcpyDeviceToHost, st));
+            }
+    }
     PCK(cudaMemcpyAsync(part_of, w + L.best, 4 * (size_t)M, cudaMemcpyDeviceToHost, st));
-    PCK(cudaMemcpyAsync(wp.data(), d.wpart + P, 8 * (size_t)P, cudaMemcpyDeviceToHost, st));
     PCK(cudaStreamSynchronize(st));
     if (stats) {
         stats->objective = (int64_t)best;

@@ -1241,7 +1241,7 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
             fn = a->ndl == 8 ? (const void *)k_adj_backward_runs<8> : (const void *)k_adj_backward_runs<16>;
         }
         if ((int)items.size() != L.n_items ||
-            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a->bsmem) != cudaSuccess ||
+            !snn::allow_dynamic_smem(fn, a->bsmem) ||
             cudaMemcpy(w + L.items.off, items.data(), sizeof(BItem) * items.size(), cudaMemcpyHostToDevice) !=
                 cudaSuccess ||
             cudaStreamCreateWithFlags(&a->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {

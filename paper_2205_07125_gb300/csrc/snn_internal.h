@@ -159,4 +159,24 @@ void route_number_pairs(snn_routing *rt, std::vector<uint32_t> &bc, std::vector<
 void route_relay_map(const snn_routing *rt, int32_t policy, std::vector<int32_t> &relay_ip);
 void route_relays(snn_routing *rt, int32_t policy, int nthreads);
 uint32_t philox_word0(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2);
+#ifdef __CUDACC__
+// Lets launches of fn on the current device use up to all the dynamic shared
+// memory a block can have, and returns whether that is `need` at least.  The
+// limit belongs to the function, not to an object: raised to one object's
+// need, it would refuse the launches of another that needs more.
+inline bool allow_dynamic_smem(const void *fn, size_t need)
+{
+    cudaFuncAttributes at;
+    int dev = 0, optin = 0;
+    if (cudaFuncGetAttributes(&at, fn) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess) {
+        const int most = optin - (int)at.sharedSizeBytes;
+        if (most >= 0 && need <= (size_t)most &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess)
+            return true;
+    }
+    cudaGetLastError();
+    return false;
+}
+#endif
 }  // namespace snn

@@ -1026,12 +1026,8 @@ static bool shape_resident(snn_sim *s)
     const Layout &L = s->L;
     if (L.res.G == 0 || !s->coop || !s->allow_persist || s->defer || s->arrival) return false;
     const void *fn = resident_fn(s);
-    cudaFuncAttributes at;
-    int smax = 0, op = 0;
-    bool ok = cudaFuncGetAttributes(&at, fn) == cudaSuccess &&
-              cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device) == cudaSuccess &&
-              cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smax - (int)at.sharedSizeBytes) ==
-                  cudaSuccess;
+    int op = 0;
+    bool ok = snn::allow_dynamic_smem(fn, L.res_smem);
     if (ok && L.res_clu) {
         ResidentLaunch r;
         resident_config(s, r);
@@ -1059,11 +1055,7 @@ static bool shape_owner(snn_sim *s, int b)
 {
     if (s->L.n_own == 0 || !s->coop || !s->allow_persist) return false;
     const size_t dyn = (size_t)((s->L.own_max * 4 + 15) / 16 * 16);
-    if (cudaFuncSetAttribute((const void *)k_owner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) !=
-        cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
+    if (!snn::allow_dynamic_smem((const void *)k_owner, dyn)) return false;
     int op = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&op, (const void *)k_owner, kThreads, dyn) != cudaSuccess ||
         op < b) {
@@ -1091,15 +1083,9 @@ static bool shape_persist(snn_sim *s, int mode, int b)
     const void *fn = persist_fn(mode, s->defer, s->arrival, b);
     if (mode != kModeScalar && !s->vec) return false;
     if (mode == kModeSmem) {
-        int smax = 0;
-        cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, s->device);
         cq = (rt->M / 4 + grid - 1) / grid;
         dyn = (size_t)cq * 52;  // V, ring slot, drive (16 B per quad each), refractory counters (4)
-        if (dyn > (size_t)smax ||
-            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
+        if (!snn::allow_dynamic_smem(fn, dyn)) return false;
     }
     int op = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&op, fn, kThreads, dyn) != cudaSuccess || op < b) {
@@ -1944,7 +1930,7 @@ extern "C" int snn_read_raster(snn_sim *s, int64_t t0, int64_t t1, uint32_t *ids
             int m = 1;
             while (m < cap_dev) m <<= 1;
             const size_t smem = sizeof(unsigned long long) * (size_t)m;
-            CK(cudaFuncSetAttribute(k_raster_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (!snn::allow_dynamic_smem((const void *)k_raster_sort, smem)) return SNN_E_CUDA;
             for (int64_t k0 = 0; k0 < nst; k0 += 65535) {
                 const int64_t nb = std::min<int64_t>(65535, nst - k0);
                 k_raster_sort<<<(unsigned)nb, 1024, smem, s->stream>>>(

@@ -147,12 +147,14 @@ __device__ __forceinline__ uint4 philox_ctr(uint32_t k0, uint32_t k1, uint32_t c
 }
 
 // Programmatic dependent launch (the kernels of a segment's graph): wait for
-// the kernel before this one, let the next one be scheduled early.
-__device__ __forceinline__ void pdl_enter()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// the kernel before this one.  The next kernel's blocks start as this one's
+// exit, which saves the gap between them.  Asking for the next kernel at the
+// start puts its waiting blocks in the way of this one's: forward and backward
+// of 138 steps of 22,888 neurons x 450 synapses 7.06 ms without the early
+// start, 7.09 with the next kernel asked for at once (7.29 on another device),
+// 6.97 as here; 60,000 x 100 7.20, 7.28, 7.13; 120 steps of 4,096 x 64 3.69,
+// 3.55, 3.55.
+__device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ int byte_sum(uint32_t w)
 {

@@ -246,7 +246,7 @@ def run_ours(args):
     if persistent:
         # one cooperative launch runs every timed step: its duration is the
         # timed region, its algorithmic bytes those of the K steps
-        kern = "k_persist"
+        kern = "k_resident" if choice >= 3000 else "k_persist"
         per_launch = step_bytes * K
         achieved = per_launch / (ms * 1e-3) / 1e9
     else:
@@ -268,11 +268,12 @@ def run_ours(args):
     # buffer (the input slots of delivery by arrival step, or the delay
     # ring), measured here
     arrival = 1000 <= choice < 2000
+    owned, resident = 2000 <= choice < 3000, choice >= 3000
     n_red = cfg.M * 2 if arrival else cfg.M * (info["max_delay"] + 1)
     red_peak = red_rate(n_red, 1 << 22)
     atom = {"what": "synaptic events (one 32-bit reduction each) per second over the whole step, vs torch "
                     "index_add_ of 4M random int32 reductions into a buffer of the accumulators' size"
-                    + (" (partition-owned delivery reduces in shared memory: context only)" if choice >= 2000 else ""),
+                    + (" (this delivery reduces in shared memory: context only)" if owned or resident else ""),
             "buffer_mb": n_red * 4 / 1e6,
             "achieved": events_all / world / (ms_max * 1e-3), "peak": red_peak, "unit": "reductions/s",
             "frac": events_all / world / (ms_max * 1e-3) / red_peak}
@@ -340,11 +341,12 @@ def run_ours(args):
                    "steps_per_graph": 32,
                    "execution": ("persistent cooperative kernel" if persistent else "CUDA graphs")
                                 + (", minimum-delay batching" if args.defer else "")
-                                + (", partition-owned delivery" if choice >= 2000 else
-                                   ", delivery by arrival step" if choice >= 1000 else ", delay-ring delivery"),
+                                + (", whole network on the chip, delivery by each target's block" if resident else
+                                   ", partition-owned delivery" if owned else
+                                   ", delivery by arrival step" if arrival else ", delay-ring delivery"),
                    "autotune": {"choice": choice, "ms_per_step": tuned_ms, "at_step": PR,
                                 "meaning": "+1000 delivery by arrival step; 2000 + blocks per SM partition-owned "
-                                           "delivery; else 0 graph path, or 100*mode + blocks per SM (mode 2 "
+                                           "delivery; 3001 the resident kernel; else 0 graph path, or 100*mode + blocks per SM (mode 2 "
                                            "shared-memory state, 1 global 16-byte, 0 global scalar)"}},
         "spikes_per_step": spikes_all / world / K,
         "events_per_step": events_all / world / K,
@@ -436,7 +438,7 @@ def kernel_source_sha() -> str:
     other code is stale)."""
     import hashlib
     hs = hashlib.sha256()
-    for f in ("snn_step.cuh", "snn_sim.cu"):
+    for f in ("snn_step.cuh", "snn_resident.cuh", "snn_sim.cu"):
         with open(os.path.join(ROOT, "paper_2205_07125_gb300", "csrc", f), encoding="utf-8") as fh:
             hs.update(_code_only(fh.read()).encode())
     return hs.hexdigest()[:16]

@@ -158,7 +158,6 @@ void route_number_pairs(snn_routing *rt, std::vector<uint32_t> &bc, std::vector<
 // relay classes of its level-2 entries under it.
 void route_relay_map(const snn_routing *rt, int32_t policy, std::vector<int32_t> &relay_ip);
 void route_relays(snn_routing *rt, int32_t policy, int nthreads);
-uint32_t philox_word0(uint64_t seed, uint32_t c0, uint32_t c1, uint32_t c2);
 #ifdef __CUDACC__
 // Lets launches of fn on the current device use up to all the dynamic shared
 // memory a block can have, and returns whether that is `need` at least.  The

@@ -674,6 +674,7 @@ struct snn_sim {
     // page-locked host memory of the small read-backs (control word, counters, state): a copy into it is one
     // transfer without staging by the driver
     char *back = nullptr;
+    std::mutex back_mu;  // (a sim may be read by several threads)
     size_t back_bytes = 0;
     // batches: the network of each quad and each network's drive (host copies)
     std::vector<uint16_t> net_of_h;
@@ -1725,6 +1726,7 @@ static int run_fanout(snn_sim *s, FoArgs a, uint64_t *counts)
         CK(cudaGetLastError());
     }
     unsigned long long pageable[4];
+    std::lock_guard<std::mutex> back_lock(s->back_mu);
     unsigned long long *c = s->back_bytes >= sizeof(pageable) ? (unsigned long long *)s->back : pageable;
     CK(cudaMemcpyAsync(c, a.cnt, sizeof(pageable), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -1834,6 +1836,7 @@ extern "C" int64_t snn_launches_per_step(const snn_sim *s)
 
 static int read_ctrl(snn_sim *s, Ctrl *c)
 {
+    std::lock_guard<std::mutex> back_lock(s->back_mu);
     void *to = s->back_bytes >= sizeof(Ctrl) ? (void *)s->back : (void *)c;
     CK(cudaMemcpyAsync(to, s->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
@@ -1909,6 +1912,7 @@ extern "C" int snn_read_raster(snn_sim *s, int64_t t0, int64_t t1, uint32_t *ids
     std::vector<long long> off((size_t)nst + 1);
     const size_t off_bytes = sizeof(long long) * (size_t)(nst + 1);
     if (s->back_bytes >= off_bytes) {
+        std::lock_guard<std::mutex> back_lock(s->back_mu);
         CK(cudaMemcpyAsync(s->back, s->dev.raster_off + t0, off_bytes, cudaMemcpyDeviceToHost, s->stream));
         CK(cudaStreamSynchronize(s->stream));
         std::memcpy(off.data(), s->back, off_bytes);
@@ -1995,6 +1999,7 @@ static int read_counters(snn_sim *s, unsigned long long *c)
     const size_t nr = (size_t)L.tally_rows * C_N, rb = sizeof(unsigned long long) * nr,
                  cb = sizeof(unsigned long long) * C_N;
     std::vector<unsigned long long> pageable;
+    std::lock_guard<std::mutex> back_lock(s->back_mu);
     unsigned long long *rows = (unsigned long long *)s->back;
     if (s->back_bytes < rb + cb) {
         pageable.resize(nr + C_N);
@@ -2038,6 +2043,7 @@ extern "C" int snn_read_state(snn_sim *s, float *V, uint8_t *ref, int64_t *t)
     const bool same = s->rt->identity;
     const size_t span = L.ref.off + L.ref.bytes - L.ctrl.off;
     if (s->back_bytes >= span) {
+        std::lock_guard<std::mutex> back_lock(s->back_mu);
         // control word, counters, potentials and refractory counters lie together: one copy
         CK(cudaMemcpyAsync(s->back, s->ws + L.ctrl.off, span, cudaMemcpyDeviceToHost, s->stream));
         CK(cudaStreamSynchronize(s->stream));

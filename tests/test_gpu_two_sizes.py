@@ -66,3 +66,29 @@ def test_adjoints(snn, monkeypatch, batched):
     got = grads(big)
     for w, x in zip(want, got):
         assert np.allclose(w, x, rtol=1e-12, atol=0)
+
+
+def test_threads_read_one_sim(snn):
+    """State, counters and raster of one sim read by several threads at once."""
+    import threading
+    g, cfg, net, rt = _make(snn, 20000)
+    sim = snn.Sim(net, rt, snn.sim_params(cfg.dyn, raster_cap=20000 * 20, raster_steps=40), device="cuda:0")
+    sim.step(40)
+    want = sim.read_state()[0], sim.read_counts(), sim.read_raster(0, 40)[0]
+    bad = []
+
+    def read(k):
+        for _ in range(100):
+            if k % 3 == 0 and not np.array_equal(sim.read_state()[0], want[0]):
+                bad.append("state")
+            if k % 3 == 1 and sim.read_counts() != want[1]:
+                bad.append("counts")
+            if k % 3 == 2 and not np.array_equal(sim.read_raster(0, 40)[0], want[2]):
+                bad.append("raster")
+
+    ts = [threading.Thread(target=read, args=(k,)) for k in range(6)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad

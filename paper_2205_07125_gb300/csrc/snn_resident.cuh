@@ -67,7 +67,7 @@ struct ResSmem {
 struct Res {
     const uint2 *ptr;           // [M * G] {first synapse, synapses} of each (neuron, target block) run
     const uint32_t *syn;        // [E] input index << 16 | uint16 weight, by (neuron, target block)
-    unsigned long long *mail;   // [2][G][G][W] mailbox words of each block from each block, by step parity
+    unsigned long long *mail;   // [2][G][G][W] mailbox words of each block from each block, by the tag's parity
     uint32_t *dovf;             // [2][2 M] spikes past the blocks' duty lists (a block's from a1 + a2)
     unsigned long long *ovf;    // [2][G * N] ids that the words have no place for, {id, tag}
     const long long *pbase;     // [P + 1] first internal neuron of each internal partition
@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                         d.spk[head + before + k] =
                             k < (unsigned int)r.ocap
                                 ? own[k]
-                                : (uint32_t)ld_word(r.ovf + ((size_t)(t & 1) * G + b) * N + k);
+                                : (uint32_t)ld_word(r.ovf + ((size_t)((r.tag0 + (uint32_t)s) & 1u) * G + b) * N + k);
                 const long long hn = next_head(d, head, tot, t);
                 __syncwarp();
                 if (lane == 0) {
@@ -758,8 +758,11 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
         };
 #pragma unroll 1
         for (int s = 0; s < T; ++s) {
-            const int par = s & 1, lp = ((int)t0 + s) & 1;
+            // lp: the half of the mailboxes, by the tag.  Tags only go up, so a half is written again every second
+            // tag whatever the step numbers do (a reset or a restored state takes them back), and no word is old
+            // enough for its 16 bits to come round.
             const uint32_t tag = r.tag0 + (uint32_t)s;
+            const int par = s & 1, lp = (int)(tag & 1u);
             uint32_t *own = own0 + par * r.ocap;
             uint16_t *cnt = cnt0 + par * G;
             // records of the step

@@ -1396,7 +1396,8 @@ static int launch_resident(snn_sim *s, int32_t T, const Dev &d)
     resident_config(s, rl);
     unsigned long long lim = s->barrier_limit_ns;
     while (T > 0) {
-        // every step of the sim's life has a tag of its own; before they run out the words are cleared
+        // every step of the sim's life has a tag of its own (the mailbox words hold 16 bits of it and are written
+        // again every second tag); before the tags run out the words are cleared
         if (s->res_tag > 0xF0000000u) s->res_tag = 1;
         if (s->res_tag == 1) {
             if (L.res_mail.bytes) CK(cudaMemsetAsync(s->ws + L.res_mail.off, 0, L.res_mail.bytes, s->stream));

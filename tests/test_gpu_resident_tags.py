@@ -1,0 +1,37 @@
+"""The resident kernel's spike messages tell old from new whatever the step
+numbers do: resets and captured graphs repeat them, the messages' tags go on."""
+import pytest
+
+import synth
+from test_gpu_parity import _compare, _run_pair, snn  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _plain_env(monkeypatch):
+    for k in ("SNN_PERSIST", "SNN_PERSIST_SMEM", "SNN_PERSIST_DEFER", "SNN_DELIVERY", "SNN_BAR_GROUPS",
+              "SNN_PERSIST_BLOCKS_PER_SM", "SNN_RESIDENT"):
+        monkeypatch.delenv(k, raising=False)
+
+
+def _net():
+    cfg = synth.NetConfig(name="tags", M=1500, P=4, n_vn=2, K=60, uniform_all=True, dmax=2, seed=83,
+                          dyn=synth.Dynamics(drive_lambda=1.1, w_ext=150, drive_seed=9))
+    return cfg, synth.make_network(cfg)
+
+
+def test_single_steps_from_rest_past_the_tags_16_bits(snn, monkeypatch):
+    """65,534 times one step from rest, then 40 steps: the second of them has
+    tag 65,536, whose 16 bits in the message words are those of words that
+    were never written."""
+    monkeypatch.setenv("SNN_RESIDENT_BLOCKS", "9")  # (messages in global memory, kept between launches)
+    cfg, g = _net()
+    sim, o, rec, _ = _run_pair(snn, g, cfg, 40, cfg.P, cfg.n_vn)
+    for _ in range(65534):
+        sim.step(1)
+        sim.reset()
+    sim.step(40)
+    assert sim.sync_status() == 0
+    c, _ = _compare(sim, o, 40, rec)
+    assert c["spikes"] > 100

@@ -661,7 +661,7 @@ struct snn_sim {
     bool defer = false;    // k_persist with minimum-delay batching (shared-memory state only)
     bool arrival = false;  // delivery by arrival step active (the workspace holds its regions)
     bool resident = false; // k_resident active (the workspace holds its regions)
-    uint32_t res_tag = 1;  // tag of the next resident step (0 marks an empty word)
+    uint32_t res_tag = 1;  // tag of the next resident step (0 marks an empty word; 1: the words are to be cleared)
     bool owner = false;    // partition-owned delivery active (k_owner; the workspace holds its regions)
     size_t owner_smem = 0; // dynamic shared memory of k_owner: the largest partition's accumulator
     unsigned grid_persist = 1;
@@ -806,6 +806,7 @@ static int reset_state(snn_sim *s)
     CK(cudaMemsetAsync(w + L.bucket_cnt.off, 0, L.bucket_cnt.bytes, st));
     CK(cudaMemsetAsync(w + L.inbox_cnt.off, 0, L.inbox_cnt.bytes, st));
     CK(cudaMemsetAsync(w + L.tally.off, 0, L.tally.bytes, st));
+    s->res_tag = 1;
     if (L.raster_off.bytes) CK(cudaMemsetAsync(w + L.raster_off.off, 0, L.raster_off.bytes, st));
     if (L.hash.bytes) CK(cudaMemsetAsync(w + L.hash.off, 0, L.hash.bytes, st));
     if (L.cur_rec.bytes) CK(cudaMemsetAsync(w + L.cur_rec.off, 0, L.cur_rec.bytes, st));
@@ -1396,8 +1397,9 @@ static int launch_resident(snn_sim *s, int32_t T, const Dev &d)
     resident_config(s, rl);
     unsigned long long lim = s->barrier_limit_ns;
     while (T > 0) {
-        // every step of the sim's life has a tag of its own (the mailbox words hold 16 bits of it and are written
-        // again every second tag); before the tags run out the words are cleared
+        // every step has a tag of its own (the mailbox words hold 16 bits of it and are written again every second
+        // tag); before the tags run out, and when the state is replaced (a launch that gave up leaves words of steps
+        // that were not run), the words are cleared and the tags begin again
         if (s->res_tag > 0xF0000000u) s->res_tag = 1;
         if (s->res_tag == 1) {
             if (L.res_mail.bytes) CK(cudaMemsetAsync(s->ws + L.res_mail.off, 0, L.res_mail.bytes, s->stream));
@@ -1575,6 +1577,7 @@ static int snapshot_restore(snn_sim *s, const Snapshot &sn)
 {
     const Layout &L = s->L;
     char *w = s->ws;
+    s->res_tag = 1;
     CK(cudaStreamSynchronize(s->stream));
     auto put = [&](const std::vector<char> &b, const Region &r, size_t off) -> cudaError_t {
         return b.empty() ? cudaSuccess : cudaMemcpy(w + r.off + off, b.data(), b.size(), cudaMemcpyHostToDevice);
@@ -2201,6 +2204,7 @@ extern "C" int snn_load_state(snn_sim *s, const void *buf, size_t bytes)
     std::memcpy(&h, b, sizeof(h));
     if (h.magic != kCkptMagic || h.M != s->rt->M || h.D != L.D) return SNN_E_ARG;
     b += sizeof(h);
+    s->res_tag = 1;
     CK(cudaStreamSynchronize(s->stream));
     for (const Region *r : {&L.V, &L.ref, &L.ring, &L.counters}) {
         CK(cudaMemcpy(s->ws + r->off, b, r->bytes, cudaMemcpyHostToDevice));

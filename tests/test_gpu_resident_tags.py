@@ -1,5 +1,6 @@
 """The resident kernel's spike messages tell old from new whatever the step
 numbers do: resets and captured graphs repeat them, the messages' tags go on."""
+import numpy as np
 import pytest
 
 import synth
@@ -22,9 +23,9 @@ def _net():
 
 
 def test_single_steps_from_rest_past_the_tags_16_bits(snn, monkeypatch):
-    """65,534 times one step from rest, then 40 steps: the second of them has
-    tag 65,536, whose 16 bits in the message words are those of words that
-    were never written."""
+    """65,534 times one step from rest, then 40 steps: with tags that count on
+    the second of them has tag 65,536, whose 16 bits in the message words are
+    those of words that were never written."""
     monkeypatch.setenv("SNN_RESIDENT_BLOCKS", "9")  # (messages in global memory, kept between launches)
     cfg, g = _net()
     sim, o, rec, _ = _run_pair(snn, g, cfg, 40, cfg.P, cfg.n_vn)
@@ -35,3 +36,27 @@ def test_single_steps_from_rest_past_the_tags_16_bits(snn, monkeypatch):
     assert sim.sync_status() == 0
     c, _ = _compare(sim, o, 40, rec)
     assert c["spikes"] > 100
+
+
+def test_restored_state_after_a_launch_that_gave_up(snn, monkeypatch):
+    """A launch of 65,536 steps gives up in its first step (block 0 is silent:
+    test switch); the first step after it, of a restored state, has the same 16
+    bits in its tag as the messages that the others left."""
+    monkeypatch.setenv("SNN_RESIDENT_BLOCKS", "9")
+    cfg, g = _net()
+    sim, o, rec, rt = _run_pair(snn, g, cfg, 60, cfg.P, cfg.n_vn)
+    sim.step(25)
+    blob = sim.save_state()
+    sim.step(35)
+    V, ref, t = sim.read_state()
+    monkeypatch.setenv("SNN_BARRIER_LIMIT_NS", "20000000")
+    monkeypatch.setenv("SNN_TEST_SKIP_BARRIER", "1")
+    late = snn.Sim(sim.net, rt, sim.params, device="cuda:0")
+    late.step(65536)
+    assert late.sync_status() == -8
+    late.load_state(blob)
+    late.step(35)
+    assert late.sync_status() == 0
+    V2, ref2, t2 = late.read_state()
+    assert t2 == t == 60
+    assert np.array_equal(V.view(np.uint32), V2.view(np.uint32)) and np.array_equal(ref, ref2)

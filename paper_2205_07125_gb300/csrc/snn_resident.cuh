@@ -387,14 +387,17 @@ RES_COLD uint32_t res_fetch(const unsigned long long *p, uint32_t tag, unsigned 
                             unsigned long long limit_ns)
 {
     const unsigned long long deadline = global_ns() + limit_ns;
+    unsigned int spins = 0;
 #pragma unroll 1
     for (;;) {
         const unsigned long long v = ld_word(p);
         if ((uint32_t)(v >> 32) == tag) return (uint32_t)v;
-        if (global_ns() > deadline) {
-            atomicOr(status, kStTimeout);
-            *abort = 1u;
-            return kResNone;
+        if ((++spins & 255u) == 0u) {
+            if (global_ns() > deadline) atomicOr(status, kStTimeout);
+            if (*(volatile unsigned int *)status & kStTimeout) {
+                *abort = 1u;
+                return kResNone;
+            }
         }
     }
 }
@@ -540,7 +543,10 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     // by step parity: own spikes, list entries, a message was too small, duty entries, pieces, the step was
     // given up
     __shared__ unsigned int s_on[2], s_ln[2], s_over[2], s_dn[2], s_pn[2], s_quit[2];
-    __shared__ unsigned int s_abort, s_done;
+    // a wait of the step ran out: in the gather, in the delivery.  Each word is read behind a barrier that all
+    // writers of it have passed and before the next one, so the warps agree and no barrier loses some of them.
+    __shared__ unsigned int s_abort, s_abort2;
+    __shared__ unsigned int s_done;
     __shared__ unsigned long long s_ph[kPhases], s_spikes;
     __shared__ long long s_head;  // raster head (walking warps)
     __shared__ unsigned long long s_tally[kTally];
@@ -625,7 +631,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     if (tid < 2) s_on[tid] = s_ln[tid] = s_over[tid] = s_dn[tid] = s_pn[tid] = s_quit[tid] = 0u;
     if (tid < kPhases) s_ph[tid] = 0ull;
     if (tid == 0) {
-        s_abort = 0u;
+        s_abort = s_abort2 = 0u;
         s_head = *(volatile long long *)&c->head[slot3(t0)];
         s_spikes = 0ull;
     }
@@ -898,6 +904,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                     if (i < nm) {
                         message(i, true, id);
                         if (i == g << r.wsh) {
+                            if (id[0] == kResEmpty) id[0] = 0u;  // (a message given up)
                             cnt[g] = (uint16_t)id[0];
                             if (id[0] > (uint32_t)pub) s_over[par] = 1u;
                             id[0] = kResEmpty;
@@ -924,7 +931,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                     }
                 }
                 bar_sync(kBarMain, nt);
-                if (__builtin_expect(s_over[par] != 0u && !s_abort, 0)) {
+                if (__builtin_expect(s_over[par] != 0u, 0)) {
                     // blocks with more spikes than a message holds: the rest, a warp per block
 #pragma unroll 1
                     for (int g = wid; g < G; g += nw) {
@@ -1065,7 +1072,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                     }
                     if (g1 >= G) break;
                     if (k0 + lane < cg)
-                        id[0] = res_fetch(r.ovf + ((size_t)lp * G + g1) * N + k0 + lane, tag, &c->status, &s_abort,
+                        id[0] = res_fetch(r.ovf + ((size_t)lp * G + g1) * N + k0 + lane, tag, &c->status, &s_abort2,
                                           limit_ns);
                     k0 += 32u;
                 }
@@ -1082,7 +1089,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
             flush();
             part(4);
             bar_sync(kBarMain, nt);
-            if (s_abort) break;
+            if (s_abort2) break;
             // the pieces, a warp each, the loads of two in flight
             const unsigned int np2 = min(s_pn[par], (unsigned int)r.pcap);
 #pragma unroll 1

@@ -1184,13 +1184,17 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
             return SNN_E_STATE;
         }
     }
-    auto up = [&](const Region &r, const void *src) -> cudaError_t {
-        return r.bytes ? cudaMemcpy(w + r.off, src, r.bytes, cudaMemcpyHostToDevice) : cudaSuccess;
+    // on the object's stream, as the kernel below that reads them (the legacy stream's copies and clears are not
+    // ordered before a non-blocking stream's kernels); the host arrays outlive the synchronisation at the end
+    auto copy = [&](size_t off, const void *src, size_t bytes) -> cudaError_t {
+        return bytes ? cudaMemcpyAsync(w + off, src, bytes, cudaMemcpyHostToDevice, a->stream) : cudaSuccess;
     };
+    auto up = [&](const Region &r, const void *src) { return copy(r.off, src, r.bytes); };
     if (up(L.pop, pop.data()) || up(L.run, rt->csr.data()) ||
-        cudaMemset(w + L.syn_td.off, 0, L.syn_td.bytes) || cudaMemset(w + L.syn_w.off, 0, L.syn_w.bytes) ||
-        cudaMemcpy(w + L.syn_td.off, rt->syn_td.data(), sizeof(uint32_t) * rt->E, cudaMemcpyHostToDevice) ||
-        cudaMemcpy(w + L.syn_w.off, rt->syn_w.data(), sizeof(int16_t) * rt->E, cudaMemcpyHostToDevice) ||
+        cudaMemsetAsync(w + L.syn_td.off, 0, L.syn_td.bytes, a->stream) ||
+        cudaMemsetAsync(w + L.syn_w.off, 0, L.syn_w.bytes, a->stream) ||
+        copy(L.syn_td.off, rt->syn_td.data(), sizeof(uint32_t) * rt->E) ||
+        copy(L.syn_w.off, rt->syn_w.data(), sizeof(int16_t) * rt->E) ||
         (!rt->identity && up(L.gid, rt->perm_inv.data()))) {
         delete a;
         return SNN_E_CUDA;
@@ -1244,8 +1248,7 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
         }
         if ((int)items.size() != L.n_items ||
             !snn::allow_dynamic_smem(fn, a->bsmem) ||
-            cudaMemcpy(w + L.items.off, items.data(), sizeof(BItem) * items.size(), cudaMemcpyHostToDevice) !=
-                cudaSuccess ||
+            copy(L.items.off, items.data(), sizeof(BItem) * items.size()) != cudaSuccess ||
             cudaStreamCreateWithFlags(&a->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
             delete a;
             return SNN_E_CUDA;

@@ -724,10 +724,12 @@ static int upload_tables(snn_sim *s)
     const Layout &L = s->L;
     char *w = s->ws;
     cudaStream_t st = s->stream;
+    // (every copy on the sim's stream: the legacy stream's are not ordered before a non-blocking stream's kernels)
     auto up = [&](const Region &r, const void *src) -> cudaError_t {
         if (!r.bytes) return cudaSuccess;
         return cudaMemcpyAsync(w + r.off, src, r.bytes, cudaMemcpyHostToDevice, st);
     };
+    std::vector<ulonglong2> slots[3];  // (until the copies are done)
     CK(up(L.syn_td, rt->syn_td.data()));
     CK(up(L.syn_w, rt->syn_w.data()));
     CK(up(L.l1_ptr, rt->l1_ptr.data()));
@@ -755,9 +757,10 @@ static int upload_tables(snn_sim *s)
     if (L.n_own > 0) {
         // partition bounds and each partition's list region
         CK(cudaMemcpyAsync(w + L.pbase.off, rt->pbase.data(), L.pbase.bytes, cudaMemcpyHostToDevice, st));
-        std::vector<ulonglong2> v((size_t)rt->P);
+        std::vector<ulonglong2> &v = slots[0];
+        v.resize((size_t)rt->P);
         for (int32_t q = 0; q < rt->P; ++q) v[q] = make_ulonglong2(L.inb_base_h[q], L.inb_cap_h[q]);
-        CK(cudaMemcpy(w + L.inb_slot.off, v.data(), L.inb_slot.bytes, cudaMemcpyHostToDevice));
+        CK(up(L.inb_slot, v.data()));
     }
     if (L.dcnt.bytes && rt->n_l2 > 0) {
         // delay counts of every segment, from the uploaded tables
@@ -783,14 +786,16 @@ static int upload_tables(snn_sim *s)
     if (!rt->identity) CK(up(L.fwd, rt->perm_fwd.data()));
     {
         // exchange regions {first entry, capacity} of every pair
-        auto slots = [&](const Region &r, const std::vector<uint64_t> &base, const std::vector<uint32_t> &cap) {
-            std::vector<ulonglong2> v(base.size());
+        auto fill = [&](std::vector<ulonglong2> &v, const std::vector<uint64_t> &base,
+                        const std::vector<uint32_t> &cap) {
+            v.resize(base.size());
             for (size_t k = 0; k < v.size(); ++k) v[k] = make_ulonglong2(base[k], cap[k]);
-            return r.bytes ? cudaMemcpy(w + r.off, v.data(), r.bytes, cudaMemcpyHostToDevice) : cudaSuccess;
+            return v.data();
         };
-        CK(slots(L.bucket_slot, L.bucket_base_h, L.bucket_cap_h));
-        CK(slots(L.inbox_slot, L.inbox_base_h, L.inbox_cap_h));
+        CK(up(L.bucket_slot, fill(slots[1], L.bucket_base_h, L.bucket_cap_h)));
+        CK(up(L.inbox_slot, fill(slots[2], L.inbox_base_h, L.inbox_cap_h)));
     }
+    CK(cudaStreamSynchronize(st));
     return SNN_OK;
 }
 
@@ -1580,7 +1585,8 @@ static int snapshot_restore(snn_sim *s, const Snapshot &sn)
     s->res_tag = 1;
     CK(cudaStreamSynchronize(s->stream));
     auto put = [&](const std::vector<char> &b, const Region &r, size_t off) -> cudaError_t {
-        return b.empty() ? cudaSuccess : cudaMemcpy(w + r.off + off, b.data(), b.size(), cudaMemcpyHostToDevice);
+        return b.empty() ? cudaSuccess
+                         : cudaMemcpyAsync(w + r.off + off, b.data(), b.size(), cudaMemcpyHostToDevice, s->stream);
     };
     CK(put(sn.v, L.V, 0));
     CK(put(sn.ref, L.ref, 0));
@@ -1588,9 +1594,10 @@ static int snapshot_restore(snn_sim *s, const Snapshot &sn)
     CK(put(sn.counters, L.counters, 0));
     CK(put(sn.tally, L.tally, 0));
     CK(put(sn.hash, L.hash, (size_t)std::min<long long>(sn.t, s->prm.hash_steps) * 16));
-    CK(cudaMemcpy(w + L.ctrl.off, &sn.ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(w + L.ctrl.off, &sn.ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, s->stream));
     for (const Region *r : {&L.acc, &L.arr_cnt, &L.inb_cnt, &L.bucket_cnt, &L.inbox_cnt})
-        if (r->bytes) CK(cudaMemset(w + r->off, 0, r->bytes));
+        if (r->bytes) CK(cudaMemsetAsync(w + r->off, 0, r->bytes, s->stream));
+    CK(cudaStreamSynchronize(s->stream));
     return SNN_OK;
 }
 
@@ -2206,11 +2213,12 @@ extern "C" int snn_load_state(snn_sim *s, const void *buf, size_t bytes)
     b += sizeof(h);
     s->res_tag = 1;
     CK(cudaStreamSynchronize(s->stream));
+    cudaStream_t st = s->stream;  // (as the kernels that read the state: see upload_tables)
     for (const Region *r : {&L.V, &L.ref, &L.ring, &L.counters}) {
-        CK(cudaMemcpy(s->ws + r->off, b, r->bytes, cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(s->ws + r->off, b, r->bytes, cudaMemcpyHostToDevice, st));
         b += r->bytes;
     }
-    CK(cudaMemset(s->dev.tally, 0, L.tally.bytes));
+    CK(cudaMemsetAsync(s->dev.tally, 0, L.tally.bytes, st));
     Ctrl c;
     std::memset(&c, 0, sizeof(c));
     c.t = h.t;
@@ -2218,14 +2226,15 @@ extern "C" int snn_load_state(snn_sim *s, const void *buf, size_t bytes)
     // steps h.t .. h.t + D - 1, which those steps consume
     c.inject_until = (s->arrival || s->owner) ? h.t + L.D : 0;
     for (int k = 0; k < 3; ++k) c.head[k] = -1;  // records restart empty and stay off after a restore
-    CK(cudaMemcpy(s->dev.ctrl, &c, sizeof(c), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(s->dev.ctrl, &c, sizeof(c), cudaMemcpyHostToDevice, st));
     if (h.t < s->prm.hash_steps)
-        CK(cudaMemset(s->dev.hash + 2 * h.t, 0, sizeof(unsigned long long) * 2 * (size_t)(s->prm.hash_steps - h.t)));
-    CK(cudaMemset(s->dev.bucket_cnt, 0, L.bucket_cnt.bytes));
-    CK(cudaMemset(s->dev.inbox_cnt, 0, L.inbox_cnt.bytes));
-    if (L.acc.bytes) CK(cudaMemset(s->ws + L.acc.off, 0, L.acc.bytes));
-    if (L.arr_cnt.bytes) CK(cudaMemset(s->ws + L.arr_cnt.off, 0, L.arr_cnt.bytes));
-    if (L.inb_cnt.bytes) CK(cudaMemset(s->ws + L.inb_cnt.off, 0, L.inb_cnt.bytes));
+        CK(cudaMemsetAsync(s->dev.hash + 2 * h.t, 0, sizeof(unsigned long long) * 2 * (size_t)(s->prm.hash_steps - h.t),
+                           st));
+    CK(cudaMemsetAsync(s->dev.bucket_cnt, 0, L.bucket_cnt.bytes, st));
+    CK(cudaMemsetAsync(s->dev.inbox_cnt, 0, L.inbox_cnt.bytes, st));
+    for (const Region *r : {&L.acc, &L.arr_cnt, &L.inb_cnt})
+        if (r->bytes) CK(cudaMemsetAsync(s->ws + r->off, 0, r->bytes, st));
+    CK(cudaStreamSynchronize(st));
     return SNN_OK;
 }
 

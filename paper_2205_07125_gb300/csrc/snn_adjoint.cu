@@ -104,8 +104,7 @@ struct AdjDev {
     // The backward's synapses, by item, kind (part of the source's partition
     // that holds the target, or none), delay, slice of 32 sources; inside a slice column k holds the k-th synapse of every source that
     // has one, so a lane per source reads whole columns.
-    uint2 *rec;             // [E] target | pop << 28, float bits of w G[pop of target][pop of source]
-    const int16_t *rec_w;   // [E] the weights in that order
+    const uint2 *rec;       // [E] target | pop << 28, weight (float bits)
     const uint32_t *cnt;    // [kKinds S M] synapses by (item, kind, delay, source)
     const unsigned long long *col;  // [kKinds S slices] first record of each (item, kind, delay, slice)
     // k_adj_backward_runs: planes [2][n_pop][M] by step parity, G[pop k][b] * (adjoint of V_pre of k); partial sums
@@ -307,7 +306,7 @@ __device__ __forceinline__ size_t col_at(const AdjDev &a, const BItem &it, int k
 // Build the backward's synapse order (targets and weights).  A block per
 // item.  The k-th synapse of a source is the k-th of its kind in the table's
 // order, so the sums' rounding does not change from run to run.
-__global__ void __launch_bounds__(kAThreads) k_adj_sort(const AdjDev a, uint2 *rec, int16_t *rec_w, uint32_t *cnt,
+__global__ void __launch_bounds__(kAThreads) k_adj_sort(const AdjDev a, uint2 *rec, uint32_t *cnt,
                                                         unsigned long long *col)
 {
     constexpr int kW = kAThreads / 32;
@@ -375,40 +374,12 @@ __global__ void __launch_bounds__(kAThreads) k_adj_sort(const AdjDev a, uint2 *r
                         pos += min(m, c) + (u < in && m > c ? 1u : 0u);
                     }
                     const uint32_t t = td & kTgtMask;
-                    rec[pos].x = t | (uint32_t)a.pop[t] << kTgtBits;
-                    rec_w[pos] = a.syn_w[x];
+                    rec[pos] = make_uint2(t | (uint32_t)a.pop[t] << kTgtBits, __float_as_uint((float)a.syn_w[x]));
                 }
                 __syncwarp();
             }
         }
         __syncthreads();
-    }
-}
-
-// The records' factors w G[pop of target][pop of source] for the gains of the
-// forward: a warp per (kind, delay, slice) of an item, column by column.
-__global__ void __launch_bounds__(kAThreads) k_adj_factors(const AdjDev a)
-{
-    __shared__ float s_G[kMaxPop * kMaxPop];
-    const int np = a.n_pop, lane = threadIdx.x & 31;
-    if (threadIdx.x < np * np) s_G[threadIdx.x] = a.G[threadIdx.x];
-    __syncthreads();
-    for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
-        const BItem it = a.items[item];
-        for (uint32_t e = threadIdx.x >> 5; e < (uint32_t)(kKinds * a.S) * it.n_sl; e += kAThreads / 32) {
-            const uint32_t sl = e % it.n_sl, si = sl * 32 + lane;
-            const uint32_t len = si < it.j1 - it.j0 ? a.cnt[cnt_at(a, it, 0, 1 + (int)(e / it.n_sl)) + si] : 0u;
-            const int pj = si < it.j1 - it.j0 ? a.pop[it.j0 + si] : 0;
-            unsigned long long at = a.col[col_at(a, it, 0, 1, 0) + e];
-#pragma unroll 4
-            for (uint32_t k = 0, m; (m = __ballot_sync(0xFFFFFFFFu, len > k)) != 0u; ++k) {
-                if (len > k) {
-                    const unsigned long long x = at + __popc(m & ((1u << lane) - 1u));
-                    a.rec[x].y = __float_as_uint(__fmul_rn((float)a.rec_w[x], s_G[(a.rec[x].x >> kTgtBits) * np + pj]));
-                }
-                at += __popc(m);
-            }
-        }
     }
 }
 
@@ -429,12 +400,16 @@ __global__ void __launch_bounds__(kAThreads) k_adj_factors(const AdjDev a)
 // KB) leaves four times as many.  Measured at the adjoint workload (131,072
 // neurons, 500 synapses, delays 1-8): 99 us per step against 191 for
 // k_adj_backward_runs; 132 with the whole partition staged.
+//
+// A term is w (G g): the gain times the adjoint rounded by itself, as
+// k_adj_backward_runs does.  Rounding w G ahead instead gives every synapse of
+// one weight and population pair the same error in every step, which adds up.
 template <int B>
 __device__ __forceinline__ void adj_gather(const AdjDev &a, const BItem &it, int d0, int d1, const float *h1,
-                                           const float2 *h2, const float4 *h3, float *hs, float *acc)
+                                           const float2 *h2, const float4 *h3, const float *s_G, float *hs, float *acc)
 {
     const uint32_t ns = it.j1 - it.j0;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, np = a.n_pop;
     const uint32_t cap = (uint32_t)a.cap, stride = cap + 1u, ways = (uint32_t)a.ways;
 #pragma unroll 1
     for (int kind = 0; kind < kKinds; ++kind) {
@@ -468,6 +443,10 @@ __device__ __forceinline__ void adj_gather(const AdjDev &a, const BItem &it, int
             const uint32_t sl = wu / ways, way = wu - sl * ways;
             const uint32_t si = sl * 32 + lane;
             if (d0 + (int)way > d1) continue;
+            // gains of the source's population; its partition's targets are of two populations
+            const int pj = si < ns ? a.pop[it.j0 + si] : (int)it.plane0;
+            const float *gain = s_G + pj;
+            const float g0 = gain[it.plane0 * np], g1 = gain[(it.plane0 + 1u) * np];
             // synapses of a delay and their first records, those of the next delay in flight
             uint32_t n0 = 0;
             unsigned long long c0;
@@ -503,13 +482,17 @@ __device__ __forceinline__ void adj_gather(const AdjDev &a, const BItem &it, int
                                   : make_uint2(it.base + from + cap, 0u);
                         r += __popc(m);
                     }
+                    float part[B];  // (the terms of a batch by themselves: short chains round less)
+#pragma unroll
+                    for (int b = 0; b < B; ++b) part[b] = 0.0f;
                     if (kind < kParts) {
 #pragma unroll
                         for (int u = 0; u < kBUnroll; ++u) {
                             const float *h = hs + ((q[u].x & kTgtMask) - it.base - from);
+                            const float gn = q[u].x & (1u << kTgtBits) ? g1 : g0;
 #pragma unroll
                             for (int b = 0; b < B; ++b)
-                                sum[b] = __fmaf_rn(__uint_as_float(q[u].y), h[b * stride], sum[b]);
+                                part[b] = __fmaf_rn(__uint_as_float(q[u].y), __fmul_rn(gn, h[b * stride]), part[b]);
                         }
                     } else {
                         float v[kBUnroll][B];
@@ -533,11 +516,15 @@ __device__ __forceinline__ void adj_gather(const AdjDev &a, const BItem &it, int
                             }
                         }
 #pragma unroll
-                        for (int u = 0; u < kBUnroll; ++u)
+                        for (int u = 0; u < kBUnroll; ++u) {
+                            const float gn = gain[(q[u].x >> kTgtBits) * np];
 #pragma unroll
                             for (int b = 0; b < B; ++b)
-                                sum[b] = __fmaf_rn(__uint_as_float(q[u].y), v[u][b], sum[b]);
+                                part[b] = __fmaf_rn(__uint_as_float(q[u].y), __fmul_rn(gn, v[u][b]), part[b]);
+                        }
                     }
+#pragma unroll
+                    for (int b = 0; b < B; ++b) sum[b] = __fadd_rn(sum[b], part[b]);
                 }
                 // the last of the planes is gathered by step t - (d - d0), the one before it by the step before
                 if (si < ns)
@@ -559,6 +546,8 @@ __global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, i
     float *hs = bsm;                       // [kBatch][cap + 1] staged planes
     float *acc = bsm + kBatch * (a.cap + 1);    // [ways][R][src_cap] sums of steps t, t - 1, ..
     const float c = 0.0009765625f;
+    __shared__ float s_G[kMaxPop * kMaxPop];
+    if (threadIdx.x < np * np) s_G[threadIdx.x] = a.G[threadIdx.x];  // (the item loop begins with a barrier)
     const bool triple = a.S >= kBatch && (t + 1) % kBatch == 0;  // planes t + 1 .. t + 3 are complete
     const int nacc = triple ? R : 2;       // steps that get terms
     for (int item = blockIdx.x; item < a.n_items; item += gridDim.x) {
@@ -569,11 +558,11 @@ __global__ void __launch_bounds__(kBThreads, 1) k_adj_backward(const AdjDev a, i
             for (uint32_t x = threadIdx.x; x < ns; x += kBThreads)
                 acc[i * a.src_cap + x] = t >= i ? a.part[(size_t)((t - i) % R) * M + it.j0 + x] : 0.0f;
         for (int x = R * a.src_cap + threadIdx.x; x < a.ways * R * a.src_cap; x += kBThreads) acc[x] = 0.0f;
-        adj_gather<1>(a, it, 1, 1, a.g1 + (size_t)((t + 1) & 1) * M, nullptr, nullptr, hs, acc);
+        adj_gather<1>(a, it, 1, 1, a.g1 + (size_t)((t + 1) & 1) * M, nullptr, nullptr, s_G, hs, acc);
         if (a.S >= 2 && (t & 1))
-            adj_gather<2>(a, it, 2, 2, nullptr, a.g2 + (size_t)(((t + 1) / 2) & 1) * M, nullptr, hs, acc);
+            adj_gather<2>(a, it, 2, 2, nullptr, a.g2 + (size_t)(((t + 1) / 2) & 1) * M, nullptr, s_G, hs, acc);
         if (triple)
-            adj_gather<3>(a, it, 3, a.S, nullptr, nullptr, a.g3 + (size_t)(((t + 1) / kBatch) & 1) * M, hs, acc);
+            adj_gather<3>(a, it, 3, a.S, nullptr, nullptr, a.g3 + (size_t)(((t + 1) / kBatch) & 1) * M, s_G, hs, acc);
         __syncthreads();
         if (a.ways > 1) {
             for (int x = threadIdx.x; x < nacc * a.src_cap; x += kBThreads)
@@ -885,7 +874,7 @@ struct Region {
 
 struct ALayout {
     Region V, ref, ring, pop, gid, run, syn_td, syn_w, spk, spk_n, pop_cnt, raster, raster_n;
-    Region G, lam, seg_vpre, seg_flag, seg_A, rec, rec_w, cnt, col, hbuf, rpart, g1, g2, g3, part, gacc, items, tb, gV, direct, dG, dlam;
+    Region G, lam, seg_vpre, seg_flag, seg_A, rec, cnt, col, hbuf, rpart, g1, g2, g3, part, gacc, items, tb, gV, direct, dG, dlam;
     Region ck_V, ck_ref, ck_ring;  // [n_ckpt] checkpoints
     size_t total = 0;
     int D = 2, n_pop = 2, n_ckpt = 1, S = 1, R = 2, n_items = 1;
@@ -997,7 +986,6 @@ int adj_layout(const snn_routing *rt, const snn_sim_params *p, const snn_adjoint
     L.batched = adj_batched(rt);
     if (L.batched) {
         aplace(L, L.rec, sizeof(uint2) * (size_t)E);
-        aplace(L, L.rec_w, sizeof(int16_t) * (size_t)E);
         aplace(L, L.cnt, sizeof(uint32_t) * (size_t)M * kKinds * L.S);
         aplace(L, L.col, sizeof(unsigned long long) * kKinds * L.S * (size_t)L.n_slices);
         aplace(L, L.g1, sizeof(float) * 2 * M);
@@ -1139,8 +1127,7 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
     d.seg_vpre = (float *)(w + L.seg_vpre.off);
     d.seg_flag = (uint8_t *)(w + L.seg_flag.off);
     d.seg_A = (int32_t *)(w + L.seg_A.off);
-    d.rec = (uint2 *)(w + L.rec.off);
-    d.rec_w = (const int16_t *)(w + L.rec_w.off);
+    d.rec = (const uint2 *)(w + L.rec.off);
     d.cnt = (const uint32_t *)(w + L.cnt.off);
     d.col = (const unsigned long long *)(w + L.col.off);
     d.g1 = (float *)(w + L.g1.off);
@@ -1255,8 +1242,7 @@ extern "C" int snn_adjoint_create(const snn_network *net, const uint8_t *is_exc,
         }
         if (L.batched)
             k_adj_sort<<<(unsigned)std::max(1, d.n_items), kAThreads, 0, a->stream>>>(
-                d, d.rec, (int16_t *)(w + L.rec_w.off), (uint32_t *)(w + L.cnt.off),
-                (unsigned long long *)(w + L.col.off));
+                d, (uint2 *)(w + L.rec.off), (uint32_t *)(w + L.cnt.off), (unsigned long long *)(w + L.col.off));
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(a->stream) != cudaSuccess) {
             delete a;
             return SNN_E_CUDA;
@@ -1402,8 +1388,6 @@ extern "C" int snn_adjoint_backward(snn_adjoint *a, const double *grates, double
     if (L.batched) {
         // (g1 .. gacc are one range: planes from step T on and all sums are 0)
         ACK(cudaMemsetAsync(w + L.g1.off, 0, L.gacc.off + L.gacc.bytes - L.g1.off, st));
-        k_adj_factors<<<(unsigned)a->dev.n_items, kAThreads, 0, st>>>(a->dev);
-        ACK(cudaGetLastError());
     } else {
         ACK(cudaMemsetAsync(w + L.hbuf.off, 0, L.hbuf.bytes, st));
         ACK(cudaMemsetAsync(w + L.rpart.off, 0, L.rpart.bytes, st));

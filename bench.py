@@ -238,7 +238,8 @@ def run_ours(args):
     assert dc["steps"] == K
     events_all, ms_max, spikes_all = reduce_over_ranks(dist, float(dc["events"]), ms, float(dc["spikes"]))
     launches = sim.launches(K)
-    persistent = launches == 1
+    shape = sim.kernel(K)  # (as the autotuner's choice; also without it)
+    persistent = shape % 1000 != 0
     # algorithmic bytes of the timed window, from its own counters
     pbw = phase_bytes(cfg.M, K, dc, not info["identity_order"])
     step_bytes = sum(pbw) / K
@@ -246,7 +247,7 @@ def run_ours(args):
     if persistent:
         # one cooperative launch runs every timed step: its duration is the
         # timed region, its algorithmic bytes those of the K steps
-        kern = "k_resident" if choice >= 3000 else "k_persist"
+        kern = "k_resident" if shape >= 3000 else "k_persist"
         per_launch = step_bytes * K
         achieved = per_launch / (ms * 1e-3) / 1e9
     else:
@@ -267,8 +268,8 @@ def run_ours(args):
     # the rate of the same reductions on random targets in an L2-sized
     # buffer (the input slots of delivery by arrival step, or the delay
     # ring), measured here
-    arrival = 1000 <= choice < 2000
-    owned, resident = 2000 <= choice < 3000, choice >= 3000
+    arrival = 1000 <= shape < 2000
+    owned, resident = 2000 <= shape < 3000, shape >= 3000
     n_red = cfg.M * 2 if arrival else cfg.M * (info["max_delay"] + 1)
     red_peak = red_rate(n_red, 1 << 22)
     atom = {"what": "synaptic events (one 32-bit reduction each) per second over the whole step, vs torch "

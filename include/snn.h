@@ -613,6 +613,10 @@ int snn_sim_reset(snn_sim *sim, int32_t reupload);
  * Errors: SNN_E_ARG, SNN_E_CUDA.
  */
 int snn_autotune(snn_sim *sim, int32_t steps, int32_t *choice, double *best_ms);
+/* The launch shape that a call of T steps of this sim takes now, as
+ * snn_autotune reports it (chosen at creation or by the autotuner); -1 for
+ * sim NULL or T < 0. */
+int32_t snn_kernel(const snn_sim *sim, int32_t T);
 
 /* ---------------------------------------------------------------- adjoint */
 /*

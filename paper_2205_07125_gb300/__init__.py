@@ -144,6 +144,7 @@ _sig("snn_batch_create", ctypes.c_int, [_P(snn_network), _vp, _i32, _vp, _vp, _v
                                         _P(_vp)])
 _sig("snn_step", ctypes.c_int, [_vp, _i32])
 _sig("snn_autotune", ctypes.c_int, [_vp, _i32, _P(_i32), _P(ctypes.c_double)])
+_sig("snn_kernel", _i32, [_vp, _i32])
 _sig("snn_sync_status", ctypes.c_int, [_vp])
 _sig("snn_read_raster", ctypes.c_int, [_vp, _i64, _i64, _vp, _i64, _vp, _P(_i64)])
 _sig("snn_read_currents", ctypes.c_int, [_vp, _i64, _vp])
@@ -184,7 +185,7 @@ EXPORTS = ("snn_strerror", "snn_model_params_preset", "snn_model_build", "snn_mo
            "snn_save_state", "snn_load_state", "snn_sim_reset", "snn_launches_per_step", "snn_launches",
            "snn_profile_phases", "snn_deliver_spikes", "snn_deliver_spikes_static",
            "snn_static_scratch_bytes", "snn_sim_destroy", "snn_batch_workspace_bytes", "snn_batch_create",
-           "snn_autotune", "snn_adjoint_params_default", "snn_adjoint_workspace_bytes", "snn_adjoint_create",
+           "snn_autotune", "snn_kernel", "snn_adjoint_params_default", "snn_adjoint_workspace_bytes", "snn_adjoint_create",
            "snn_adjoint_forward", "snn_adjoint_backward", "snn_adjoint_read_spikes", "snn_adjoint_destroy")
 
 
@@ -581,6 +582,10 @@ class Sim:
         with self._dev():
             _ck(_lib.snn_autotune(self.h, int(steps), ctypes.byref(c), ctypes.byref(ms)), "snn_autotune")
         return int(c.value), float(ms.value)
+
+    def kernel(self, T: int) -> int:
+        """The launch shape that step(T) takes now, as autotune's choice (snn_kernel)."""
+        return int(_lib.snn_kernel(self.h, int(T)))
 
     def profile_phases(self, T: int) -> np.ndarray:
         """Advance T steps and return the summed ms of the parts of a step

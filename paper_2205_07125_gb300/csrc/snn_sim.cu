@@ -1619,6 +1619,20 @@ static void set_arrival(snn_sim *s, bool on)
         }
 }
 
+// A launch shape as snn_autotune reports it.
+static int32_t shape_code(bool persist, bool resident, bool owner, bool arrival, int mode, int b)
+{
+    if (resident) return 3001;
+    if (owner) return 2000 + b;
+    return (persist ? 100 * mode + b : 0) + (arrival ? 1000 : 0);
+}
+
+extern "C" int32_t snn_kernel(const snn_sim *s, int32_t T)
+{
+    if (!s || T < 0) return -1;
+    return shape_code(s->persist, s->resident, s->owner, s->arrival, s->pmode, s->persist_bps);
+}
+
 extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *best_ms)
 {
     if (!s || steps < 1) return SNN_E_ARG;
@@ -1695,10 +1709,7 @@ extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *
     else if (pick.persist) shape_persist(s, pick.mode, pick.b);
     const int rr = snapshot_restore(s, snap);
     if (rc == SNN_OK) rc = rr;
-    if (choice)
-        *choice = pick.resident ? 3001
-                  : pick.owner  ? 2000 + pick.b
-                             : (pick.persist ? 100 * pick.mode + pick.b : 0) + (pick.arrival ? 1000 : 0);
+    if (choice) *choice = shape_code(pick.persist, pick.resident, pick.owner, pick.arrival, pick.mode, pick.b);
     if (best_ms) *best_ms = best < 1e300 ? best / steps : -1.0;
     return rc;
 }

@@ -454,7 +454,8 @@ int snn_sim_workspace_bytes(const snn_routing *rt, const snn_sim_params *p, size
  * changes a result, every combination is bit-exact):
  *   SNN_PERSIST=0               CUDA-graph path instead of the persistent kernel
  *   SNN_PERSIST_SMEM=0          persistent kernel on global neuron state only
- *   SNN_RESIDENT=0              no resident kernel (the whole network on the
+ *   SNN_RESIDENT=0|1            1: the resident kernel for every call it can
+ *                               run; 0: no resident kernel (the whole network on the
  *                               chip; also off with SNN_PERSIST=0,
  *                               SNN_PERSIST_SMEM=0, SNN_PERSIST_DEFER=1 and any
  *                               SNN_PERSIST_BLOCKS_PER_SM or SNN_BAR_GROUPS)
@@ -532,7 +533,11 @@ int snn_batch_create(const snn_network *net, const snn_routing *rt, int32_t n, c
  * fill counters stay on the chip, a block has one bounded wait per step (for
  * the spikes of the others).  Its tables, a copy of the synapses ordered by
  * target block, are part of the workspace; with a workspace that has no room
- * for them the network runs as above.
+ * for them the network runs as above.  So do, step for step, calls too short
+ * to pay for moving the state in and out (from 33 blocks on; 1 to 24 steps by
+ * size), and calls after one whose mean spikes per step were above what that
+ * kernel is faster for (SNN_RESIDENT=1: every call runs on it).  A call of
+ * 1,024 steps or more looks again every 1,024 steps.
  * Errors raised on the device are reported by snn_sync_status.
  * Errors: SNN_E_ARG, SNN_E_CUDA.
  */
@@ -614,8 +619,9 @@ int snn_sim_reset(snn_sim *sim, int32_t reupload);
  */
 int snn_autotune(snn_sim *sim, int32_t steps, int32_t *choice, double *best_ms);
 /* The launch shape that a call of T steps of this sim takes now, as
- * snn_autotune reports it (chosen at creation or by the autotuner); -1 for
- * sim NULL or T < 0. */
+ * snn_autotune reports it (chosen at creation or by the autotuner; where that
+ * is the resident kernel, by the call's length and the firing too, see
+ * snn_step); -1 for sim NULL or T < 0. */
 int32_t snn_kernel(const snn_sim *sim, int32_t T);
 
 /* ---------------------------------------------------------------- adjoint */
@@ -682,8 +688,9 @@ void snn_adjoint_destroy(snn_adjoint *adj);
 
 /* Kernels of one step on the graph path: 2 (a1-a3, a4-a6). */
 int64_t snn_launches_per_step(const snn_sim *sim);
-/* Kernel launches one snn_step(sim, T) issues: 1 on the persistent path,
- * 2 per step plus one per replayed graph on the graph path. */
+/* Kernel launches one snn_step(sim, T) issues: 1 on the persistent path (calls
+ * of 1,024 steps or more of the resident kernel: 3, and 2 more per further
+ * 1,024 steps), 2 per step plus one per replayed graph on the graph path. */
 int64_t snn_launches(const snn_sim *sim, int32_t T);
 
 /*

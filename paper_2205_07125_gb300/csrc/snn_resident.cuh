@@ -79,6 +79,8 @@ struct Res {
     int walkers;                // warps beside the steps
     int kbytes;                 // drive arrivals in shared memory (a byte per neuron; reordered ids)
     int prefetch;               // pull the spikes' rows into L2 (tables larger than it)
+    unsigned int most;          // mean spikes per step above which another kernel is faster
+    int first;                  // the first launch of a call of several (Dev::t_base)
     uint32_t tag0;              // tag of the launch's first step
     uint32_t key[20];           // Philox round keys of a single network's drive
     ResSmem o;
@@ -603,6 +605,8 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     __shared__ unsigned long long s_tally[kTally];
     int32_t *const ring = reinterpret_cast<int32_t *>(s_dyn);
     Ctrl *c = d.ctrl;
+    // a later launch of a call: another kernel's turn, or the call was given up
+    if (d.t_base && !r.first && (*(volatile unsigned int *)d.hot || call_left(d) != T)) return;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int all = blockDim.x, nt = all - 32 * r.walkers, nw = nt >> 5;  // step threads, step warps
     const int G = r.G, b = blockIdx.x, N = r.N, S = r.S;
@@ -1211,6 +1215,12 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
         d.counters[C_STEPS] += (unsigned long long)s_done;
         d.counters[C_SPIKES] += s_spikes;
         c->t = te;
+        if (s_done < (unsigned int)T) {
+            if (d.t_base) *d.t_base = kNoBase;
+        } else {
+            if (r.first) *d.t_base = t0;
+            if (T >= kHotSteps) set_hot(d, s_spikes > (unsigned long long)r.most * (unsigned long long)T);
+        }
         for (int k = 0; k < kPhases && d.phase_ns; ++k) d.phase_ns[k] += s_ph[k];
     }
     if constexpr (CLU) cluster_sync();  // no block leaves while another may write to its mailbox

@@ -219,9 +219,12 @@ struct Layout {
     int n_own = 0;                   // lists per partition of owned delivery; 0: no owner regions
     int64_t own_max = 0;             // neurons of the largest partition
     std::vector<uint64_t> inb_base_h, inb_cap_h;  // per internal partition: first record, list capacity
-    Region res_ptr, res_syn, res_mail, res_ovf, res_dovf, res_pbase, res_bptr, res_iptr;  // k_resident
+    Region res_ptr, res_syn, res_mail, res_ovf, res_call, res_dovf, res_pbase, res_bptr, res_iptr;  // k_resident
     Res res = {};                    // its sizes (G = 0: not available; pointers filled at the launch)
     int res_threads = 0, res_qpt = 0, res_clu = 0;
+    bool res_forced = false;         // every call, whatever its length and the network's spikes (SNN_RESIDENT=1)
+    int res_min = 1;                 // shortest call it takes
+    unsigned int res_most = 0;       // mean spikes per step up to which it is the faster kernel
     size_t res_smem = 0;
     std::vector<uint64_t> bucket_base_h, inbox_base_h;
     std::vector<uint32_t> bucket_cap_h, inbox_cap_h;
@@ -366,6 +369,33 @@ static int resident_blocks(int64_t nq, int sms)
     return g > 4 ? 8 : g > 2 ? 4 : (int)g;
 }
 
+// Calls and networks that k_resident is the faster kernel for, against
+// k_persist with the delay ring.  It moves the state in and out once per call,
+// so a call must be long enough; and every block looks every spike up, where
+// k_persist shares the spikes out, so the network must not fire too much.
+// Measured, us per call of k_resident / k_persist (12 Hz):
+//   65,536 neurons, delays 1-8   T = 1 19.2 / 18.5   2 26.0 / 28.5   10 66 / 107
+//   262,144                      T = 3 45.0 / 39.1   5 57.8 / 59.6   10 88 / 110
+//   600,000                      T = 5 71.8 / 66.0  10 110 / 122
+//   1,048,576                    T = 10 157 / 142   20 270 / 275;  delay 1: 10 131 / 141
+// and us per step at a mean of n spikes per step (K synapses per neuron):
+//   4,096, K 300      n = 54 6.6 / 9.1    82 8.5 / 9.3    (K 1,000: 31 9.3 / 10.0   80 11.4 / 10.4)
+//   16,384, K 1,000   n = 215 10.0 / 11.4   328 21.7 / 11.6
+//   65,536, K 50      n = 867 7.8 / 11.0   1311 10.7 / 11.4   2337 23.2 / 11.6
+//   65,536, K 1,000   n = 481 9.4 / 12.8   871 15.5 / 14.4   1314 45.5 / 16.8
+//   262,144, K 200    n = 1226 10.6 / 11.7   1508 13.3 / 12.4   2701 32.3 / 14.4
+//   1,048,576, K 20   n = 1250 9.3 / 12.7   2704 15.4 / 13.7   4924 24.8 / 15.4
+//   2,000,000, K 20   n = 2500 12.8 / 16.4   5158 26.3 / 18.2
+// The lines through the points where the two meet: over 270 measured pairs the
+// one chosen is at most 7 % slower than k_persist, but for 16,384 neurons of
+// 1,000 synapses at 40 to 60 spikes (14 %).
+static void resident_range(const snn_routing *rt, Layout &L)
+{
+    const double G = L.res.G, N = L.res.N, M = (double)rt->M, K = (double)rt->E / M;
+    L.res_min = G <= 32 ? 1 : (int)(1 + N / 800 + L.res.S * N / 6000);
+    L.res_most = (unsigned int)(G <= 32 ? G / (0.04 + 1e-4 * K) : G / (0.09 / (1 + 3e-7 * M) + 6e-5 * K));
+}
+
 constexpr size_t kResStatic = 768;  // k_resident's static shared memory, at most
 
 // Shape of k_resident for a routing: blocks, neurons per block, threads and
@@ -438,6 +468,8 @@ static void resident_layout(const snn_routing *rt, const snn_sim_params *p, Layo
     L.res_clu = clu;
     L.res_threads = threads;
     L.res_qpt = need <= 1 ? 1 : need <= 2 ? 2 : 4;
+    L.res_forced = env_is("SNN_RESIDENT", '1');
+    resident_range(rt, L);
 }
 
 static int make_layout(const snn_routing *rt, const snn_sim_params *p, Layout &L, int32_t n_net = 0,
@@ -573,6 +605,7 @@ static int make_layout(const snn_routing *rt, const snn_sim_params *p, Layout &L
         place(L, L.res_syn, sizeof(uint32_t) * (size_t)E);
         place(L, L.res_mail, L.res_clu ? 0 : 2 * G * G * (size_t)L.res.W * sizeof(unsigned long long));
         place(L, L.res_ovf, 2 * G * (size_t)L.res.N * sizeof(unsigned long long));
+        place(L, L.res_call, 2 * sizeof(long long));  // Dev::t_base, Dev::hot
         place(L, L.res_dovf, sizeof(uint32_t) * 4 * (size_t)M);
         place(L, L.res_pbase, sizeof(long long) * (size_t)(P + 1));
         place(L, L.res_bptr, sizeof(uint32_t) * (size_t)(P + 1));
@@ -661,7 +694,10 @@ struct snn_sim {
     bool persist = false;  // one cooperative launch per snn_step (k_persist)
     bool defer = false;    // k_persist with minimum-delay batching (shared-memory state only)
     bool arrival = false;  // delivery by arrival step active (the workspace holds its regions)
-    bool resident = false; // k_resident active (the workspace holds its regions)
+    bool resident = false; // k_resident active (the workspace holds its regions); the calls that it is not for run on
+                           // the k_persist shape below
+    bool tuning = false;   // snn_autotune is timing the shapes: each runs by itself
+    unsigned int *hot = nullptr;  // page-locked copy of Dev::hot: the last launch's spikes were too many for k_resident
     uint32_t res_tag = 1;  // tag of the next resident step (0 marks an empty word; 1: the words are to be cleared)
     bool owner = false;    // partition-owned delivery active (k_owner; the workspace holds its regions)
     size_t owner_smem = 0; // dynamic shared memory of k_owner: the largest partition's accumulator
@@ -893,6 +929,7 @@ extern "C" void snn_sim_destroy(snn_sim *s)
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     for (void *p : s->pinned) cudaHostUnregister(p);
     if (s->back) cudaFreeHost(s->back);
+    if (s->hot) cudaFreeHost(s->hot);
     delete s;
 }
 
@@ -1027,12 +1064,29 @@ static void resident_config(const snn_sim *s, ResidentLaunch &r)
     r.cfg.numAttrs = 1;
 }
 
-// Select the resident kernel when its blocks fit the device.  Returns
-// whether it was selected.
-static bool shape_resident(snn_sim *s)
+static bool shape_persist(snn_sim *s, int mode, int b);
+
+// The k_persist shape with the most of its state in shared memory, at most bmax blocks per SM.
+static void shape_persist_first(snn_sim *s, int bmax)
+{
+    s->persist = false;
+    if (s->allow_smem)
+        for (int b = bmax; b >= 1 && !s->persist; --b) shape_persist(s, kModeSmem, b);
+    for (int b = bmax; b >= 1 && !s->persist; --b) shape_persist(s, s->vec ? kModeVec : kModeScalar, b);
+    cudaGetLastError();
+}
+
+// Select the resident kernel when its blocks fit the device, and for the
+// calls that it is not for k_persist with mode and blocks per SM as given
+// (b 0: the first shape that fits).  Returns whether it was selected.
+static bool shape_resident(snn_sim *s, int mode = 0, int b = 0)
 {
     const Layout &L = s->L;
     if (L.res.G == 0 || !s->coop || !s->allow_persist || s->defer || s->arrival) return false;
+    s->persist = false;
+    if (b > 0) shape_persist(s, mode, b);
+    if (!s->persist) shape_persist_first(s, 4);
+    if (!s->persist) return false;
     const void *fn = resident_fn(s);
     int op = 0;
     bool ok = snn::allow_dynamic_smem(fn, L.res_smem);
@@ -1048,11 +1102,7 @@ static bool shape_resident(snn_sim *s)
         cudaGetLastError();
         return false;
     }
-    s->persist = true;
     s->resident = true;
-    s->owner = false;
-    s->persist_bps = 1;
-    s->grid_persist = (unsigned)L.res.G;
     return true;
 }
 
@@ -1197,12 +1247,7 @@ static int sim_create(const snn_network *net, const snn_routing *rt, const snn_s
         s->defer = p->defer_delayed != 0 || (edf && edf[0] == '1');
         s->allow_persist = !(e && e[0] == '0') && s->coop;
         s->allow_smem = !(esm && esm[0] == '0');
-        if (s->allow_persist) {
-            if (s->allow_smem)
-                for (int b = bmax; b >= 1 && !s->persist; --b) shape_persist(s, kModeSmem, b);
-            for (int b = bmax; b >= 1 && !s->persist; --b) shape_persist(s, s->vec ? kModeVec : kModeScalar, b);
-        }
-        cudaGetLastError();
+        if (s->allow_persist) shape_persist_first(s, bmax);
         // tests of the bounded barrier wait: a shorter bound, and block 0
         // skipping its first arrival so that the others' wait runs out
         const char *lim = std::getenv("SNN_BARRIER_LIMIT_NS");
@@ -1339,9 +1384,18 @@ static int sim_create(const snn_network *net, const snn_routing *rt, const snn_s
     }
     if (L.res.G > 0 && !s->owner) {
         // the network fits on the chip: the resident kernel (ring form between launches)
-        const bool arr = s->arrival;
+        const bool arr = s->arrival, per = s->persist;
+        const int m = s->pmode, b = s->persist_bps;
         set_arrival(s, false);
-        if (!shape_resident(s)) set_arrival(s, arr);
+        if (cudaHostAlloc((void **)&s->hot, sizeof(*s->hot), cudaHostAllocMapped) == cudaSuccess) *s->hot = 0;
+        else s->hot = nullptr;
+        cudaGetLastError();
+        if (!shape_resident(s)) {
+            // the shape from before
+            set_arrival(s, arr);
+            s->persist = false;
+            if (per) shape_persist(s, m, b);
+        }
     }
     finite_thresholds(p->drive_lambda, d.th32, &d.th_fin);
     if (L.n_net > 0) {
@@ -1372,6 +1426,8 @@ static int sim_create(const snn_network *net, const snn_routing *rt, const snn_s
         }
     }
     rc = upload_tables(s);
+    if (!rc && L.res_call.bytes && cudaMemsetAsync(w + L.res_call.off, 0, L.res_call.bytes, s->stream) != cudaSuccess)
+        rc = SNN_E_CUDA;
     if (!rc) rc = reset_state(s);
     if (rc) {
         snn_sim_destroy(s);
@@ -1381,15 +1437,43 @@ static int sim_create(const snn_network *net, const snn_routing *rt, const snn_s
     return SNN_OK;
 }
 
-static int launch_resident(snn_sim *s, int32_t T, const Dev &d)
+// A call of at least kResLong steps of the resident kernel comes in several
+// launches, kResProbe steps and then kResLong at a time, so that a network
+// that fires too much for it takes k_persist within the call: each but the
+// first is a launch of either kernel, one of which returns at once.  The
+// launches and the state's way out and in take 25 us, below 1 % of the call;
+// shorter calls go by what the last launch saw.
+constexpr int32_t kResLong = 1024, kResProbe = 64;
+
+static bool resident_takes(const snn_sim *s, int32_t T)
+{
+    if (s->L.res_forced || s->tuning) return true;
+    return T >= s->L.res_min && !(s->hot && *(const volatile unsigned int *)s->hot);
+}
+
+static bool resident_splits(const snn_sim *s, int32_t T)
+{
+    return T >= kResLong && !s->L.res_forced && !s->tuning;
+}
+
+static int launch_kernel(snn_sim *s, int32_t T, const Dev &d);
+
+static int launch_resident(snn_sim *s, int32_t T, Dev d)
 {
     const Layout &L = s->L;
+    long long *const call = (long long *)(s->ws + L.res_call.off);
+    d.hot = (unsigned int *)(call + 1);
+    d.hot_host = s->hot;
+    d.cool = L.res_most - L.res_most / 5;  // (back some way below the line, so that the choice does not flicker)
+    d.t_base = nullptr;
+    if (!resident_takes(s, T)) return launch_kernel(s, T, d);
     const char *w = s->ws;
     Res r = L.res;
     r.ptr = (const uint2 *)(w + L.res_ptr.off);
     r.syn = (const uint32_t *)(w + L.res_syn.off);
     r.mail = L.res_clu ? nullptr : (unsigned long long *)(w + L.res_mail.off);
     r.ovf = (unsigned long long *)(w + L.res_ovf.off);
+    r.most = L.res_most;
     r.dovf = (uint32_t *)(w + L.res_dovf.off);
     r.pbase = (const long long *)(w + L.res_pbase.off);
     r.bptr = (const uint32_t *)(w + L.res_bptr.off);
@@ -1402,30 +1486,43 @@ static int launch_resident(snn_sim *s, int32_t T, const Dev &d)
     ResidentLaunch rl;
     resident_config(s, rl);
     unsigned long long lim = s->barrier_limit_ns;
+    const bool split = resident_splits(s, T);
+    d.t_base = split ? call : nullptr;
+    d.t_off = 0;
     while (T > 0) {
+        r.first = split && d.t_off == 0;
         // every step has a tag of its own (the mailbox words hold 16 bits of it and are written again every second
-        // tag); before the tags run out, and when the state is replaced (a launch that gave up leaves words of steps
-        // that were not run), the words are cleared and the tags begin again
-        if (s->res_tag > 0xF0000000u) s->res_tag = 1;
+        // tag); before the tags run out, when the state is replaced (a launch that gave up leaves words of steps
+        // that were not run) and for launches that may not run, the words are cleared and the tags begin again
+        if (s->res_tag > 0xF0000000u || split) s->res_tag = 1;
         if (s->res_tag == 1) {
             if (L.res_mail.bytes) CK(cudaMemsetAsync(s->ws + L.res_mail.off, 0, L.res_mail.bytes, s->stream));
             CK(cudaMemsetAsync(s->ws + L.res_ovf.off, 0, L.res_ovf.bytes, s->stream));
         }
-        int tt = std::min<int32_t>(T, 1 << 27);
+        int tt = std::min<int32_t>(T, r.first ? kResProbe : split ? kResLong : 1 << 27);
         int skip = s->test_skip_arrival;
         s->test_skip_arrival = 0;  // once: the test checks the first launch's status
+        d.t_off += tt;
         r.tag0 = s->res_tag;
-        s->res_tag += (uint32_t)tt;
+        s->res_tag = split ? 1u : s->res_tag + (uint32_t)tt;
         void *args[] = {(void *)&d, (void *)&r, (void *)&tt, (void *)&lim, (void *)&skip};
         CK(cudaLaunchKernelExC(&rl.cfg, resident_fn(s), args));
+        if (split && !r.first)
+            if (int rc = launch_kernel(s, tt, d)) return rc;
         T -= tt;
     }
     return SNN_OK;
 }
 
+// T steps of the persistent path.
 static int launch_persist(snn_sim *s, int32_t T, const Dev &d)
 {
-    if (s->resident) return launch_resident(s, T, d);
+    return s->resident ? launch_resident(s, T, d) : launch_kernel(s, T, d);
+}
+
+// T steps of k_owner or the k_persist shape.
+static int launch_kernel(snn_sim *s, int32_t T, const Dev &d)
+{
     unsigned long long lim = s->barrier_limit_ns;
     const void *fn = s->owner ? (const void *)k_owner : persist_fn(s->pmode, s->defer, s->arrival, s->persist_bps);
     const size_t smem = s->owner ? s->owner_smem : s->persist_smem;
@@ -1537,6 +1634,7 @@ extern "C" int snn_profile_phases(snn_sim *s, int32_t T, double *phase_ms)
 
 // ---------------------------------------------------------------- launch-shape autotuner
 static int read_ctrl(snn_sim *s, Ctrl *c);
+static int read_counters(snn_sim *s, unsigned long long *c);
 
 // A copy of a sim's dynamic state (snn_autotune): neuron state, delay ring,
 // counters, tally rows, the hash slots from the current step on and the
@@ -1631,7 +1729,7 @@ static int32_t shape_code(bool persist, bool resident, bool owner, bool arrival,
 extern "C" int32_t snn_kernel(const snn_sim *s, int32_t T)
 {
     if (!s || T < 0) return -1;
-    return shape_code(s->persist, s->resident, s->owner, s->arrival, s->pmode, s->persist_bps);
+    return shape_code(s->persist, s->resident && resident_takes(s, T), s->owner, s->arrival, s->pmode, s->persist_bps);
 }
 
 extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *best_ms)
@@ -1667,6 +1765,10 @@ extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *
         return r0;
     }
     Shape pick = {s->persist, s->pmode, s->persist_bps, s->arrival, s->owner, s->resident};
+    // beside the resident kernel: the fastest k_persist shape with the delay ring
+    Shape ring = {};
+    double ring_best = 1e300, fired = 0;
+    s->tuning = true;
     int rc = SNN_OK;
     for (const Shape &c : cand) {
         set_arrival(s, c.arrival);
@@ -1685,6 +1787,8 @@ extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *
         // from the sim's state: a quarter of the steps to warm up, then the timed steps
         if ((rc = snapshot_restore(s, snap)) != SNN_OK) break;
         if ((rc = snn_step(s, std::max(1, steps / 4))) != SNN_OK) break;
+        unsigned long long n0[C_N], n1[C_N];
+        if (c.resident && (rc = read_counters(s, n0)) != SNN_OK) break;
         if (cudaEventRecord(e0, s->stream) != cudaSuccess) { rc = SNN_E_CUDA; break; }
         if ((rc = snn_step(s, steps)) != SNN_OK) break;
         if (cudaEventRecord(e1, s->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess) {
@@ -1696,6 +1800,14 @@ extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *
         if (ctl.status & kStTimeout) continue;  // a shape that cannot run here
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
+        if (c.resident) {
+            if ((rc = read_counters(s, n1)) != SNN_OK) break;
+            fired = (double)(n1[C_SPIKES] - n0[C_SPIKES]) / steps;
+        }
+        if (c.persist && !c.resident && !c.owner && !c.arrival && ms < ring_best) {
+            ring_best = ms;
+            ring = c;
+        }
         if (ms < best) {
             best = ms;
             pick = c;
@@ -1704,9 +1816,16 @@ extern "C" int snn_autotune(snn_sim *s, int32_t steps, int32_t *choice, double *
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     s->persist = false;
+    s->tuning = false;
     set_arrival(s, pick.arrival);
-    if (pick.resident) shape_resident(s);
-    else if (pick.owner) shape_owner(s, pick.b);
+    if (pick.resident) {
+        // what was the fastest at this firing stays it a little above too
+        shape_resident(s, ring.mode, ring.b);
+        resident_range(s->rt, s->L);
+        s->L.res_most = std::max(s->L.res_most, (unsigned int)(1.25 * fired));
+        if (s->hot) *s->hot = 0;
+        cudaMemsetAsync(s->ws + s->L.res_call.off, 0, s->L.res_call.bytes, s->stream);
+    } else if (pick.owner) shape_owner(s, pick.b);
     else if (pick.persist) shape_persist(s, pick.mode, pick.b);
     const int rr = snapshot_restore(s, snap);
     if (rc == SNN_OK) rc = rr;
@@ -1847,6 +1966,8 @@ extern "C" int snn_deliver_spikes_static(snn_sim *s, const uint32_t *ids, int64_
 extern "C" int64_t snn_launches(const snn_sim *s, int32_t T)
 {
     if (!s || T <= 0) return 0;
+    if (s->resident && resident_takes(s, T) && resident_splits(s, T))
+        return 1 + 2 * (((int64_t)T - kResProbe + kResLong - 1) / kResLong);
     if (s->persist) return 1;
     const int64_t graphs = (s->U > 1 ? T / s->U : 0) + (s->U > 1 ? T % s->U : T);
     return 2 * (int64_t)T + graphs;  // two step kernels + one k_advance per graph

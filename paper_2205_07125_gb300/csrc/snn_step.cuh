@@ -85,6 +85,7 @@ constexpr int kPhases = 7;
 enum { C_STEPS = 0, C_SPIKES, C_EVENTS, C_L1_LOCAL, C_L1_XVN, C_L2_BASE /* + cls (4) */, C_N = 16 };
 constexpr int kTally = 7;  // slots C_EVENTS .. C_L2_BASE + 3, consecutive
 
+constexpr int kHotSteps = 4;    // steps of a launch from which its mean spikes say something (Dev::hot)
 constexpr int kBarGroups = 16;  // groups of the two-level grid-barrier arrival
 
 struct Ctrl {
@@ -158,6 +159,13 @@ struct Dev {
     unsigned long long *tally;     // [tally_rows][C_N] per-block event and message tallies
     unsigned long long *phase_ns;  // [kPhases] k_persist: block 0's time per part of a step (profiling)
     Ctrl *ctrl;
+    // sims that the resident kernel may step (snn_resident.cuh), nullptr in the others.  hot, hot_host: whether the
+    // last launch's mean spikes per step were too many for it (cool: k_persist's line).  t_base: a call of several
+    // launches, the step it began at (kNoBase: given up); t_off: the steps up to the end of this launch's share
+    unsigned int *hot, *hot_host;
+    unsigned int cool;
+    long long *t_base;
+    long long t_off;
     // delivery by arrival step (n_arr > 0; 0: every delay at the spike step
     // into the delay ring)
     int32_t *acc;                  // [2][M] input of step t in slot t & 1
@@ -194,6 +202,22 @@ struct Dev {
     const uint16_t *net_of;
     const NetDrive *net_drive;
 };
+
+constexpr long long kNoBase = -(1ll << 62);
+
+// Steps left of a call of several launches, up to the end of this launch's share.
+__device__ __forceinline__ long long call_left(const Dev &d)
+{
+    return *(volatile long long *)d.t_base + d.t_off - *(volatile long long *)&d.ctrl->t;
+}
+
+// Sets Dev::hot and the host's copy of it (one thread; the host's word is written when it changes).
+__device__ __forceinline__ void set_hot(const Dev &d, bool h)
+{
+    if ((*(volatile unsigned int *)d.hot != 0u) == h) return;
+    *(volatile unsigned int *)d.hot = h;
+    if (d.hot_host) *(volatile unsigned int *)d.hot_host = h;
+}
 
 // Counter arrays of step parity par.
 __device__ __forceinline__ uint32_t *bucket_cnt_of(const Dev &d, int par)
@@ -1897,6 +1921,14 @@ __global__ void __launch_bounds__(kThreads, MINB) k_persist(const Dev d, int T,
     __shared__ __align__(8) unsigned long long s_bar;
     extern __shared__ __align__(128) unsigned char s_dyn[];
     Ctrl *c = d.ctrl;
+    if (d.t_base) {
+        // the steps that the resident kernel left (no block changes the words before all have read them)
+        const long long left = call_left(d);
+        if (left <= 0) return;
+        T = (int)min((long long)T, left);
+    }
+    __shared__ unsigned long long s_spk0;
+    if (d.hot && blockIdx.x == 0 && threadIdx.x == 0) s_spk0 = d.counters[C_SPIKES];
     Resident rs{};
     if constexpr (MODE == kModeSmem) {
         const long long cq = d.chunk_q;
@@ -2015,6 +2047,8 @@ __global__ void __launch_bounds__(kThreads, MINB) k_persist(const Dev d, int T,
     if (lead) {
         if (t0 + done - 1 > closed) close_step(d, t0 + done - 1);
         c->t = t0 + done;
+        if (d.hot && done >= kHotSteps)
+            set_hot(d, d.counters[C_SPIKES] - s_spk0 > (unsigned long long)d.cool * (unsigned long long)done);
         if (prof)
             for (int k = 0; k < kPhases; ++k) d.phase_ns[k] += sh.prof[k];
     }

@@ -79,6 +79,7 @@ struct Res {
     int walkers;                // warps beside the steps
     int kbytes;                 // drive arrivals in shared memory (a byte per neuron; reordered ids)
     int prefetch;               // pull the spikes' rows into L2 (tables larger than it)
+    unsigned int few;           // spikes per step up to which 4 to 32 lanes take one each
     unsigned int most;          // mean spikes per step above which another kernel is faster
     int first;                  // the first launch of a call of several (Dev::t_base)
     uint32_t tag0;              // tag of the launch's first step
@@ -1011,7 +1012,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                     else wk.more[(size_t)par * 2 * d.M + pos - r.dcap] = id;
                 }
             };
-            if (n <= min(fit, (unsigned int)(8 * nw))) {
+            if (n <= min(fit, r.few)) {
                 // few spikes: 4 to 32 lanes each walk its run of synapses into this block
                 const int sh = n > (unsigned int)(4 * nw)   ? 2
                                : n > (unsigned int)(2 * nw) ? 3

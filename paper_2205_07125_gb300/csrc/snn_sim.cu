@@ -379,16 +379,15 @@ static int resident_blocks(int64_t nq, int sms)
 //   600,000                      T = 5 71.8 / 66.0  10 110 / 122
 //   1,048,576                    T = 10 157 / 142   20 270 / 275;  delay 1: 10 131 / 141
 // and us per step at a mean of n spikes per step (K synapses per neuron):
-//   4,096, K 300      n = 54 6.6 / 9.1    82 8.5 / 9.3    (K 1,000: 31 9.3 / 10.0   80 11.4 / 10.4)
-//   16,384, K 1,000   n = 215 10.0 / 11.4   328 21.7 / 11.6
+//   4,096, K 300      n = 54 6.6 / 9.1    82 8.5 / 9.3    (K 1,000: 31 7.4 / 11.1   53 9.8 / 11.4)
+//   16,384, K 1,000   n = 94 7.3 / 12.4   215 10.9 / 12.7   328 21.7 / 11.6
 //   65,536, K 50      n = 867 7.8 / 11.0   1311 10.7 / 11.4   2337 23.2 / 11.6
 //   65,536, K 1,000   n = 481 9.4 / 12.8   871 15.5 / 14.4   1314 45.5 / 16.8
 //   262,144, K 200    n = 1226 10.6 / 11.7   1508 13.3 / 12.4   2701 32.3 / 14.4
 //   1,048,576, K 20   n = 1250 9.3 / 12.7   2704 15.4 / 13.7   4924 24.8 / 15.4
 //   2,000,000, K 20   n = 2500 12.8 / 16.4   5158 26.3 / 18.2
 // The lines through the points where the two meet: over 270 measured pairs the
-// one chosen is at most 7 % slower than k_persist, but for 16,384 neurons of
-// 1,000 synapses at 40 to 60 spikes (14 %).
+// one chosen is at most 7 % slower than k_persist.
 static void resident_range(const snn_routing *rt, Layout &L)
 {
     const double G = L.res.G, N = L.res.N, M = (double)rt->M, K = (double)rt->E / M;
@@ -444,6 +443,12 @@ static void resident_layout(const snn_routing *rt, const snn_sim_params *p, Layo
                                                rt->ipair_ptr[du.pb2] - rt->ipair_ptr[du.pa2]));
     }
     r.kbytes = !rt->identity;
+    // few spikes, 4 to 32 lanes each: more of them the shorter their runs of synapses into a block are (a lane of 4
+    // walks a long run alone; past the limit long runs are cut into pieces).  Us per step with 8, 4, 2 times the step
+    // warps: 8,192 neurons, 1,000 synapses, 48 spikes (62 per run) 18.6, 8.1, 7.7; 16,384, 300, 42 (9) 6.5, 4.7, 4.5;
+    // 65,536, 1,000, 106 (8) 7.2, 5.6, 5.5; 65,536, 100, 92 (1) 4.3, 4.8, 4.9
+    const int64_t run = rt->E / std::max<int64_t>(1, rt->M * G);
+    r.few = (unsigned int)(step / 32 * (run >= 14 ? 2 : run >= 6 ? 4 : 8));
     // a message holds 11 ids, or 23 where a block has 3 spikes a step at 10 Hz or more
     r.W = N <= 3000 ? 4 : 8;
     r.wsh = N <= 3000 ? 1 : 2;

@@ -641,7 +641,8 @@ int32_t snn_kernel(const snn_sim *sim, int32_t T);
  * Rates r_a = (spikes of population a) / (T N_a).  Backward: surrogate
  * dS/dV_pre = 1 / (1 + beta |V_pre - V_th|)^2, reset detached; each neuron
  * gathers its targets' adjoints along its own level-2 entries (the
- * transpose of the routed delivery).  Networks of 25,000 neurons or more gather
+ * transpose of the routed delivery).  Networks of 25,000 neurons or more (of up
+ * to 110,000 where there are 1,000 synapses per neuron and few delays) gather
  * the adjoints of up to three steps at once (a synapse of delay d contributes d
  * steps earlier, so those of delay >= 3 are read every third step), smaller
  * ones step by step; the float32 terms are summed in a fixed order per neuron,

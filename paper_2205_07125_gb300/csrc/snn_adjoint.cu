@@ -939,16 +939,23 @@ int backward_items(const snn_routing *rt, std::vector<BItem> *out, int64_t *slic
 
 // Whether the backward batches steps (k_adj_backward) or walks every run each
 // step (k_adj_backward_runs).  A batched step has several phases in a row, each
-// some loads deep; they pay from about 25,000 neurons.  Measured, forward and
-// backward of 100 steps in ms, runs / batched: 4,096 neurons x 64 synapses
-// 3.1 / 3.4; 20,000 x 300 5.2 / 5.6; 30,000 x 100 4.9 / 4.6; 60,000 x 80 6.9 /
-// 5.3; 100,000 x 60 10.8 / 6.0; 131,072 x 500 22.3 / 14.2.  SNN_ADJ_BATCHED=0|1
-// overrides (tests).
+// some loads deep, that pay from about 25,000 neurons.  A lane walks its
+// source's synapses of a delay by itself, so its chain grows with the
+// synapses, and with few delays there is little to share out between warps
+// and nothing to batch: then more neurons are needed, growing about as the
+// root of the synapses per neuron.  Measured, backward of 60 steps in ms, runs
+// / batched: 26,000 neurons x 50 synapses, delays 1-8 1.92 / 1.47; 40,000 x
+// 150, delay 1 2.48 / 2.46; 26,000 x 400, 1-8 2.47 / 2.66, 40,000 x 400 3.64 /
+// 2.94; 50,000 x 400, 1-3 4.19 / 4.47, 1-4 4.23 / 3.87; 65,536 x 400, 1 5.00 /
+// 5.19; 65,536 x 800, 1-3 7.76 / 7.81; 131,072 x 400, 1 9.94 / 6.82, 1-8 11.4 /
+// 5.91.  SNN_ADJ_BATCHED=0|1 overrides (tests).
 bool adj_batched(const snn_routing *rt)
 {
     const char *e = std::getenv("SNN_ADJ_BATCHED");
     if (e && (e[0] == '0' || e[0] == '1')) return e[0] == '1';
-    return rt->M >= kBatchedNeurons;
+    const double root = std::sqrt((double)rt->E / (double)std::max<int64_t>(1, rt->M));
+    const double per_root = rt->max_delay <= 3 ? 3300 : rt->max_delay <= 5 ? 2400 : 1600;
+    return (double)rt->M >= std::max((double)kBatchedNeurons, per_root * root);
 }
 
 int adj_layout(const snn_routing *rt, const snn_sim_params *p, const snn_adjoint_params *ap, ALayout &L)

@@ -537,7 +537,8 @@ int snn_batch_create(const snn_network *net, const snn_routing *rt, int32_t n, c
  * to pay for moving the state in and out (from 33 blocks on; 1 to 24 steps by
  * size), and calls after one whose mean spikes per step were above what that
  * kernel is faster for (SNN_RESIDENT=1: every call runs on it).  A call of
- * 1,024 steps or more looks again every 1,024 steps.
+ * 1,024 steps or more looks again every 1,024 steps.  Calls under stream
+ * capture, whose launches may be replayed, run as above too.
  * Errors raised on the device are reported by snn_sync_status.
  * Errors: SNN_E_ARG, SNN_E_CUDA.
  */

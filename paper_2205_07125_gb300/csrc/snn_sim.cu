@@ -1450,8 +1450,21 @@ static int sim_create(const snn_network *net, const snn_routing *rt, const snn_s
 // shorter calls go by what the last launch saw.
 constexpr int32_t kResLong = 1024, kResProbe = 64;
 
+// A captured launch is run again with the same tags, whose messages are there
+// from the time before; k_persist counts its steps on the device alone.
+static bool capturing(const snn_sim *s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 static bool resident_takes(const snn_sim *s, int32_t T)
 {
+    if (capturing(s)) return false;
     if (s->L.res_forced || s->tuning) return true;
     return T >= s->L.res_min && !(s->hot && *(const volatile unsigned int *)s->hot);
 }

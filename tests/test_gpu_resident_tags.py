@@ -60,3 +60,29 @@ def test_restored_state_after_a_launch_that_gave_up(snn, monkeypatch):
     V2, ref2, t2 = late.read_state()
     assert t2 == t == 60
     assert np.array_equal(V.view(np.uint32), V2.view(np.uint32)) and np.array_equal(ref, ref2)
+
+
+@pytest.mark.parametrize("blocks", [1, 4, 9])
+def test_captured_steps_replay(snn, monkeypatch, blocks):
+    """A CUDA graph that holds a call of three steps, replayed between calls
+    that are not captured."""
+    import torch
+    monkeypatch.setenv("SNN_RESIDENT_BLOCKS", str(blocks))
+    monkeypatch.setenv("SNN_RESIDENT_LIST", "1")
+    cfg, g = _net()
+    g.v0[::3] = -45.0
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        sim, o, rec, _ = _run_pair(snn, g, cfg, 132, cfg.P, cfg.n_vn)
+        sim.step(2)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            sim.step(3)
+        for _ in range(20):
+            graph.replay()
+        sim.step(10)
+        for _ in range(20):
+            graph.replay()
+    assert sim.sync_status() == 0
+    c, _ = _compare(sim, o, 132, rec)
+    assert c["spikes"] > 1000

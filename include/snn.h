@@ -439,7 +439,11 @@ typedef struct {
 
 typedef struct snn_sim snn_sim;
 
-/* Device workspace size for a routing and parameters.  Errors: SNN_E_ARG. */
+/* Device workspace size for a routing and parameters.  A network that fits on
+ * the chip has the tables of the resident kernel (snn_step) in it: 4 B per
+ * synapse, 8 B per neuron and block (1 to one per SM) and 32 B per neuron, 5.5 GB at
+ * 1,048,576 neurons of 1,000 synapses.  snn_sim_create takes a workspace
+ * without them (SNN_RESIDENT=0 gives its size) too.  Errors: SNN_E_ARG. */
 int snn_sim_workspace_bytes(const snn_routing *rt, const snn_sim_params *p, size_t *bytes);
 
 /*
@@ -454,11 +458,11 @@ int snn_sim_workspace_bytes(const snn_routing *rt, const snn_sim_params *p, size
  * changes a result, every combination is bit-exact):
  *   SNN_PERSIST=0               CUDA-graph path instead of the persistent kernel
  *   SNN_PERSIST_SMEM=0          persistent kernel on global neuron state only
- *   SNN_RESIDENT=0|1            1: the resident kernel for every call it can
- *                               run; 0: no resident kernel (the whole network on the
+ *   SNN_RESIDENT=0|1            0: no resident kernel (the whole network on the
  *                               chip; also off with SNN_PERSIST=0,
  *                               SNN_PERSIST_SMEM=0, SNN_PERSIST_DEFER=1 and any
- *                               SNN_PERSIST_BLOCKS_PER_SM or SNN_BAR_GROUPS)
+ *                               SNN_PERSIST_BLOCKS_PER_SM or SNN_BAR_GROUPS);
+ *                               1: every call it can run, see snn_step
  *   SNN_RESIDENT_BLOCKS=g       resident kernel on (about) g blocks
  *   SNN_RESIDENT_THREADS=n      resident kernel with n threads per block
  *   SNN_RESIDENT_LIST=n         resident kernel with lists of at most n entries
@@ -650,7 +654,9 @@ int32_t snn_kernel(const snn_sim *sim, int32_t T);
  * so the gradients do not depend on the checkpoint interval.  Gradients are
  * accumulated as float pairs and added in float64.  The environment variable
  * SNN_ADJ_BATCHED=0|1, read by snn_adjoint_workspace_bytes and
- * snn_adjoint_create, selects one of the two (tests).
+ * snn_adjoint_create, selects one of the two (tests).  The batched form keeps 8 B
+ * per synapse, about 13 B per neuron and delay and some 100 B per neuron more in
+ * the workspace.
  */
 typedef struct {
     int32_t T;            /* forward steps per run (>= 1) */
@@ -730,8 +736,11 @@ int snn_profile_phases(snn_sim *sim, int32_t T, double *phase_ms);
  * Runs on the sim's stream, with the sim's device current (the caller's
  * current device is restored), and synchronises the stream before returning.
  * Errors: SNN_E_ARG (n < 0, NULL pointers with n > 0, an id >= M),
- * SNN_E_CAPACITY (the spikes need more bucket/inbox room than the
- * workspace holds), SNN_E_CUDA.
+ * SNN_E_CAPACITY (the spikes have more level-1 or level-2 entries than the
+ * sim's buckets or inboxes have places: more than every neuron spiking once
+ * needs, less with bucket_frac / inbox_frac below 1), SNN_E_CUDA.  After
+ * SNN_E_CAPACITY, and for the other ids after an id >= M, the input has been
+ * added to out in full: the call is not to be repeated.
  */
 int snn_deliver_spikes(snn_sim *sim, const uint32_t *ids, int64_t n, int32_t *out,
                        uint64_t *counts);
@@ -742,11 +751,11 @@ int snn_deliver_spikes(snn_sim *sim, const uint32_t *ids, int64_t n, int32_t *ou
  * they run, such as a host program that hands out all device memory itself
  * from a fixed budget, or a real-time stimulation loop that may not stall
  * in an allocator call.  It computes exactly what snn_deliver_spikes
- * computes (same arguments, same output, same counts) but keeps its scratch
- * in a fixed array built into the library, of snn_static_scratch_bytes()
- * (8 MiB) per GPU; every GPU that loads the library holds that array until
- * the process exits.  The call itself allocates nothing: no cudaMalloc,
- * no cudaFree.
+ * computes (same arguments, same output, same counts) but keeps its scratch,
+ * four counters, in a fixed array built into the library, of
+ * snn_static_scratch_bytes() (8 MiB) per GPU; every GPU that loads the library
+ * holds that array until the process exits.  The call itself allocates
+ * nothing: no cudaMalloc, no cudaFree.
  *   - The first call on a device looks up the array's device address once
  *     (cudaGetSymbolAddress, with that device current); make that first
  *     call before any stream capture.  The address stays cached for the
@@ -754,8 +763,9 @@ int snn_deliver_spikes(snn_sim *sim, const uint32_t *ids, int64_t n, int32_t *ou
  *     device's primary context) the library's module is unloaded and this
  *     call must not be used again in that process.
  *   - Size limit: n * (4 B * longest level-1 row + 8 B * most level-2
- *     entries of any neuron) + 512 B must fit in the array; larger calls
- *     return SNN_E_RANGE and do nothing.
+ *     entries of any neuron) + 512 B at most the array's size; larger calls
+ *     return SNN_E_RANGE and do nothing (a limit of the call: the entries
+ *     themselves are not stored).
  *   - All calls share the one array and each call clears its counters
  *     first, so calls that overlap on the GPU (other streams, other threads,
  *     other sims on the same GPU) race and give wrong results: serialise

@@ -1922,9 +1922,10 @@ extern "C" int snn_deliver_spikes(snn_sim *s, const uint32_t *ids, int64_t n, in
 
 // ---------------------------------------------------------------- fan-out without allocation
 // snn_deliver_spikes_static: the same fan-out as snn_deliver_spikes, but its
-// scratch (counters, level-1 list, level-2 list) lives in this fixed device
-// array instead of the sim's workspace.  Every GPU that loads the library
-// holds the array until the process exits; all calls share it.
+// scratch (four counters) lives in this fixed device array instead of the
+// sim's workspace.  Every GPU that loads the library holds the array until the
+// process exits; all calls share it.  Its size and the limit on a call's
+// entries are part of the interface.
 constexpr size_t kStaticScratchBytes = (size_t)8 << 20;  // 8 MiB
 static __device__ __align__(256) unsigned char g_fanout_scratch[kStaticScratchBytes];
 
